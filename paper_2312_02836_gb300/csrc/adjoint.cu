@@ -29,7 +29,7 @@
 
 #include "blob.h"
 #include "adjoint.cuh"
-#include "coop.cuh"
+#include "coop_adjoint.cuh"
 #include "device.cuh"
 #include "host.h"
 #include "../../include/netburn.h"
@@ -99,15 +99,18 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams A) {
   }
 }
 
-// One warp per zone.  With A.blob_in_smem > 1 the warp's Newton-loop arrays
-// and its adjoint arrays sit in shared memory after the (optional) blob
-// copy: [forward hot | adjoint] per warp, adj_doubles of adjoint arrays.
+// One zone per team of P threads.  With C.smem the team's Newton-loop arrays
+// and its adjoint arrays sit in shared memory after the (optional) blob copy,
+// C.stride doubles per team; else everything is in the workspace.
 struct CoopAdj {
-  int smem;           // arrays in shared memory
-  int adj_doubles;    // adjoint arrays per zone
+  int smem, stride;
+  TeamAdj a;
 };
 
-__global__ void __launch_bounds__(256, 1) k_adjoint_coop(AdjParams A, CoopAdj C) {
+template <int P, int S, int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, MINB) 
+    k_adjoint_coop(const __grid_constant__ AdjParams A, const __grid_constant__ CoopAdj C,
+                   const __grid_constant__ BlobHeader H) {
   extern __shared__ __align__(16) unsigned char sm[];
   const unsigned char* blob = A.blob;
   if (A.blob_in_smem) {
@@ -117,42 +120,67 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_coop(AdjParams A, CoopAdj C)
     __syncthreads();
     blob = sm;
   }
-  const WNet t = make_wnet<32>(blob, threadIdx.x & 31);
-  const int wib = threadIdx.x >> 5;
-  const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
-  const long long fwd = t.g.lane_doubles;
-  CWS w;
-  AWST<CV> a;
+  unsigned char* rest = sm + (A.blob_in_smem ? A.blob_bytes : 0);
+  const TNet<P, S> t(BlobDims(blob, H), reinterpret_cast<unsigned long long*>(rest));
+  const int tib = threadIdx.x / P;
+  const long long team = (long long)blockIdx.x * (blockDim.x / P) + tib;
+  const int thot = H.thot, tcold = H.tcold;
+  double *hot, *cold;
   if (C.smem) {
-    double* hot = reinterpret_cast<double*>(sm + (A.blob_in_smem ? A.blob_bytes : 0)) +
-                  (size_t)wib * (t.g.hot_doubles + C.adj_doubles);
-    w = make_cws(t.g, hot, A.ws + warp * (fwd - t.g.hot_doubles));
-    a = make_aws_at<CV>(A, hot + t.g.hot_doubles - fwd, 1);
+    hot = reinterpret_cast<double*>(rest + team_scratch_bytes(P)) + (size_t)tib * C.stride;
+    cold = A.ws + team * tcold;
   } else {
-    double* base = A.ws + warp * A.lane_doubles;
-    w = make_cws(t.g, base, base + t.g.hot_doubles);
-    a = make_aws_at<CV>(A, base, 1);
+    hot = A.ws + team * (thot + C.a.total + tcold);
+    cold = hot + thot + C.a.total;
   }
+  CWS w = make_cws(H, hot, cold);
+  const TAWS a = make_taws(C.a, hot + thot);
+  AdjZone Zs;
+  bool active = false;
   for (;;) {
-    unsigned long long c = 0;
-    if (t.lane == 0) c = atomicAdd(A.queue, 1ull);
-    c = __shfl_sync(kFullMask, c, 0);
-    if (c >= (unsigned long long)A.Z) break;
-    AdjZone Zs;
-    Zs.z = A.order ? (long long)A.order[c] : (long long)c;
-    Zs.rs = 1;
-    Zs.re = 0;
-    Zs.lo = 1;
-    bool done = adj_init(t, Zs, w, a, A);
-    while (!done) done = Zs.rs <= Zs.re ? adj_replay(t, Zs, w, a, A) : adj_step(t, Zs, w, a, A);
-    adj_finish(t, Zs, a, A);
-    __syncwarp();
+    bool done;
+    if (!active) {
+      unsigned long long c = 0;
+      if (t.lane == 0) c = atomicAdd(A.queue, 1ull);
+      c = t.bcast(c);
+      if (c >= (unsigned long long)A.Z) break;
+      Zs.z = A.order ? (long long)A.order[c] : (long long)c;
+      Zs.rs = 1;
+      Zs.re = 0;
+      Zs.lo = 1;
+      done = adj_init(t, Zs, w, a, A);
+    } else if (Zs.rs <= Zs.re) {
+      done = adj_replay(t, Zs, w, a, A);
+    } else {
+      done = adj_step(t, Zs, w, a, A);
+    }
+    active = !done;
+    if (done) {
+      adj_finish(t, Zs, a, A);
+      t.sync();
+    }
   }
 }
 
 __global__ void k_zone_index(int32_t* idx, long long Z) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < Z) idx[i] = (int32_t)i;
+}
+
+// offsets of a team's adjoint arrays for K cotangent sets
+void team_layout(const BlobHeader& h, int K, int stride, int S, TeamAdj* a) {
+  int off = 0;
+  auto take = [&](long long cnt) { const int o = off; off += (int)cnt; return o; };
+  a->lam = take((long long)HMAX * K * h.n);
+  a->ee = take(HMAX * K);
+  a->gr = take((long long)K * h.R);
+  a->gt = take(K);
+  a->mu = take((long long)K * team_mu(h.n, S));
+  a->de = take(h.n);
+  a->seg = take((long long)stride * h.n);
+  a->ce = take(K);
+  a->vs = take(h.self_heating ? 0 : (long long)(S > 0 ? 1 : K) * h.R);
+  a->total = (off + 1) & ~1;
 }
 
 }  // namespace
@@ -217,36 +245,53 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
   int tpb, in_smem;
   size_t dyn;
   long long blocks;
-  CoopAdj C{0, (int)(A.lane_doubles - h.lane_doubles)};
-  size_t per_unit;   // global workspace per lane (lane kernel) or warp (coop)
+  CoopAdj C;
+  std::memset(&C, 0, sizeof(C));
+  const size_t scratch = team_scratch_bytes(64);
+  auto team_fn = &k_adjoint_coop<64, 32, 64, 4>;
+  size_t per_unit;   // global workspace per lane (lane kernel) or team (coop)
   if (kernel == NB_KERNEL_COOP) {
-    // per warp in shared memory: the forward hot arrays and the adjoint's
-    const size_t warp_b = ((size_t)h.hot_doubles + C.adj_doubles) * sizeof(double);
-    int wpb = o.threads_per_block > 0 ? o.threads_per_block / 32 : 0;
-    if (o.threads_per_block % 32 != 0 || wpb > 8) return NB_E_ARG;
-    in_smem = 0;
-    C.smem = o.ws_in_shared != 0 && warp_b <= net->smem_optin;
-    if (wpb == 0) {
-      wpb = 4;
-      if (C.smem) while (wpb > 1 && (size_t)wpb * warp_b > net->smem_optin) --wpb;
+    // per team in shared memory: the forward hot arrays and the adjoint's
+    const int S = 32;
+    team_layout(h, K, tp->dev.stride, S, &C.a);
+    C.stride = h.thot + C.a.total;
+    const size_t team_b = (size_t)C.stride * sizeof(double);
+    // an explicit block of several zones has to fit with one zone per warp
+    const int warps = o.threads_per_block / 32;
+    if (o.threads_per_block % 32 != 0 || warps > 8) return NB_E_ARG;
+    const size_t warp_b = ((size_t)h.hot_doubles + A.lane_doubles - h.lane_doubles) * sizeof(double);
+    if (warps > 0 && o.ws_in_shared != 0 && warp_b <= net->smem_optin &&
+        warps * warp_b > net->smem_optin)
+      return NB_E_TOO_LARGE;
+    C.smem = o.ws_in_shared != 0 && team_b + scratch <= net->smem_optin;
+    // Threads of a team (a block each): four warps while the longest zone
+    // sets the time (up to 8 zones an SM: 1,024 zones of the 48-species
+    // network take 226, 220, 184 ms with 1, 2, 4 warps), else two (4,096
+    // zones: 315, 243, 411 ms); where two zones' arrays don't fit an SM's
+    // shared memory, eight
+    if (C.smem && 2 * (team_b + 1024) > net->smem_optin) {
+      tpb = 256;
+      team_fn = &k_adjoint_coop<256, 32, 256, 1>;
+    } else if (C.smem && Z <= 8LL * net->sm_count) {
+      tpb = 128;
+      team_fn = &k_adjoint_coop<128, 32, 128, 2>;
+    } else {
+      tpb = 64;
+      team_fn = &k_adjoint_coop<64, 32, 64, 4>;
     }
-    if (o.blob_in_shared != 0 && blob_b <= 96 * 1024 &&
-        blob_b + (C.smem ? wpb * warp_b : 0) <= net->smem_optin)
-      in_smem = 1;
-    dyn = (in_smem ? blob_b : 0) + (C.smem ? wpb * warp_b : 0);
-    if (dyn > net->smem_optin) return NB_E_TOO_LARGE;
-    tpb = wpb * 32;
-    CK(cudaFuncSetAttribute(k_adjoint_coop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    in_smem = o.blob_in_shared != 0 && blob_b <= 96 * 1024 &&
+              blob_b + scratch + (C.smem ? team_b : 0) <= net->smem_optin;
+    dyn = (in_smem ? blob_b : 0) + scratch + (C.smem ? team_b : 0);
+    CK(cudaFuncSetAttribute((const void*)team_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)dyn));
     int occ = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_adjoint_coop, tpb, dyn));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
     if (occ < 1) return NB_E_TOO_LARGE;
     const int bps = std::max(1, std::min(o.blocks_per_sm > 0 ? o.blocks_per_sm : occ, occ));
     blocks = (long long)bps * net->sm_count;
-    const long long needed = (Z + wpb - 1) / wpb;
-    if (blocks > needed) blocks = needed;
-    per_unit = (C.smem ? (size_t)(h.lane_doubles - h.hot_doubles) : (size_t)A.lane_doubles) * 8;
-    const size_t need = (size_t)blocks * wpb * per_unit;
+    if (blocks > Z) blocks = Z;
+    per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
+    const size_t need = (size_t)blocks * per_unit;
     int rc = nb::ensure((void**)&net->ws_adj, &net->ws_adj_bytes, std::max<size_t>(need, 256));
     if (rc) return rc;
   } else {
@@ -297,7 +342,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
   }
   CK(cudaMemsetAsync(A.queue, 0, sizeof(unsigned long long), st));
   if (kernel == NB_KERNEL_COOP)
-    k_adjoint_coop<<<(unsigned)blocks, tpb, dyn, st>>>(A, C);
+    team_fn<<<(unsigned)blocks, tpb, dyn, st>>>(A, C, h);
   else
     k_adjoint<<<(unsigned)blocks, tpb, dyn, st>>>(A);
   CK(cudaGetLastError());

@@ -84,11 +84,6 @@ NB_HD __forceinline__ AWS make_aws(const AdjParams& A, double* lane_base) {
   return make_aws_at<LV>(A, lane_base, WS_LANES);
 }
 
-// the compiled network of either network type
-NB_HD __forceinline__ const Net& net_of(const Net& t) { return t; }
-template <class NT>
-NB_HD __forceinline__ const Net& net_of(const NT& t) { return t.g; }
-
 // Set up the recomputation of the block holding step s_hi: load its history
 // window (records q0, q0-1, .. with q0 = the block's start) from the tape
 // into the forward history ring, as the forward burn held it before step
@@ -193,61 +188,81 @@ NB_HD inline bool adj_replay(const NT& t, AdjZone& Zs, WT& w, const AT& a, const
 
 // d edot / dx into a.de (needs w.dt at x): per species, its derivative terms
 // in increasing order (the order a scatter over the terms adds them in)
-template <class NT, class WT, class AT>
-NB_HD __forceinline__ void edot_gradient(const NT& t, const WT& w, const AT& a) {
-  const Net& g = net_of(t);
-  if constexpr (is_coop<NT>::value) {
-    for (int j = vbeg(t); j < t.N; j += vstep(t)) {
-      double acc = 0.0;
-      for (int e = t.dej_ptr[j]; e < t.dej_ptr[j + 1]; ++e) {
-        const int d = t.dej_d[e];
-        acc += g.Q[g.dt_r[d]] * w.dt[d];
-      }
-      a.de[j] = acc;
-    }
-    if (t.sh) {
-      double acc = 0.0;
-      for (int r = vbeg(t); r < t.R; r += vstep(t)) acc = fma(g.Q[r], w.dt[g.nd + r], acc);
-      acc = vsum(t, acc);
-      if (vlead(t)) a.de[t.N] = acc;
-    }
-  } else {
-    for (int i = 0; i < t.n; ++i) a.de[i] = 0.0;
-    for (int d = 0; d < g.nd; ++d) a.de[g.dt_j[d]] += g.Q[g.dt_r[d]] * w.dt[d];
-    if (t.sh) {
-      double acc = 0.0;
-      for (int r = 0; r < t.R; ++r) acc = fma(g.Q[r], w.dt[g.nd + r], acc);
-      a.de[t.N] = acc;
-    }
+template <class WT, class AT>
+NB_HD __forceinline__ void edot_gradient(const Net& t, const WT& w, const AT& a) {
+  for (int i = 0; i < t.n; ++i) a.de[i] = 0.0;
+  for (int d = 0; d < t.nd; ++d) a.de[t.dt_j[d]] += t.Q[t.dt_r[d]] * w.dt[d];
+  if (t.sh) {
+    double acc = 0.0;
+    for (int r = 0; r < t.R; ++r) acc = fma(t.Q[r], w.dt[t.nd + r], acc);
+    a.de[t.N] = acc;
   }
-  vsync(t);
 }
 
-// v <- M^-T v with the factored LU of either network type
-NB_HD __forceinline__ void solve_MT_of(const Net& t, const LV& lu, const LV& v) {
-  tri_solve(t.tfw, t.tfw_s, t.tfw_c, t.n, lu, v);
-  tri_solve(t.tbw, t.tbw_s, t.tbw_c, t.n, lu, v);
+// alpha_j of recorded step s (times s, s-1, ..)
+NB_HD __forceinline__ void adj_alpha(const Net&, const AdjParams& A, long long z, int s, int kk,
+                                     double h, step_alpha<Net>& alpha) {
+  double tau[KMAX + 1];
+#pragma unroll
+  for (int j = 0; j <= KMAX; ++j) tau[j] = (j <= kk) ? sched_ptr(A, z, s - j)[0] : 0.0;
+  bdf_alpha(kk, tau, h, alpha.a);
 }
-template <class NT, class LUV, class V>
-NB_HD __forceinline__ void solve_MT_of(const NT& t, const LUV& lu, const V& v) {
-  solve_MT(t, lu, v);
+
+// the K cotangents of one reverse step, one after the other: mu_q =
+// M^-T (lam_q + e_q h / alpha_0 d edot/dx), its share of the older points'
+// cotangents and of the rate gradient
+template <class WT, class AT>
+NB_HD __forceinline__ void adj_sets(const Net& t, const WT& w, const AT& a, int K, int kk,
+                                    int sl, const int* sj, const step_alpha<Net>& alpha, double h,
+                                    double ia0, double icv) {
+  const int n = t.n;
+  for (int q = 0; q < K; ++q) {
+    const int lo = (sl * K + q) * n;
+    const double es = a.ee[sl * K + q];
+    const double ce = es * h * ia0;
+    for (int i = 0; i < n; ++i) {
+      double v = a.lam[lo + i];
+      if (t.hasE) v = fma(ce, a.de[i], v);
+      a.mu[i] = v;
+      a.lam[lo + i] = 0.0;
+    }
+    a.ee[sl * K + q] = 0.0;
+    tri_solve(t.tfw, t.tfw_s, t.tfw_c, n, w.lu, a.mu);
+    tri_solve(t.tbw, t.tbw_s, t.tbw_c, n, w.lu, a.mu);
+#pragma unroll
+    for (int j = 1; j <= KMAX; ++j) {
+      if (j > kk) continue;
+      const int lj = (sj[j] * K + q) * n;
+      const double ma = -alpha[j];
+      for (int i = 0; i < n; ++i) a.lam[lj + i] = fma(ma, a.mu[i], a.lam[lj + i]);
+      if (t.hasE) a.ee[sj[j] * K + q] = fma(-es * ia0, alpha[j], a.ee[sj[j] * K + q]);
+    }
+    const double muT = t.sh ? a.mu[t.N] * icv : 0.0;
+    double gt = 0.0;
+    for (int r = 0; r < t.R; ++r) {
+      double acc = 0.0;
+      for (int e = t.rg_ptr[r]; e < t.rg_ptr[r + 1]; ++e)
+        acc = fma(t.rg_c[e], a.mu[t.rg_i[e]], acc);
+      const double Qr = t.Q[r];
+      acc = fma(muT, Qr, acc);
+      const double v = w.rr[r] * fma(h, acc, ce * Qr);
+      a.gr[q * t.R + r] += v;
+      if (!t.sh) gt = fma(v, w.g[r], gt);
+    }
+    a.gt[q] += gt;
+  }
 }
 
 // reverse one step; returns true when the zone is done
 template <class NT, class WT, class AT>
 NB_HD inline bool adj_step(const NT& t, AdjZone& Zs, WT& w, const AT& a, const AdjParams& A) {
-  const Net& g = net_of(t);
   const long long z = Zs.z;
   const int n = t.n, N = t.N, K = A.K, s = Zs.s;
   const double* ss = sched_ptr(A, z, s);
   const int kk = A.tape.ord[(size_t)z * A.tape.cap + s];
   const double h = ss[1];
-  double tau[KMAX + 1];
-  tau[0] = ss[0];
-#pragma unroll
-  for (int j = 1; j <= KMAX; ++j) tau[j] = (j <= kk) ? sched_ptr(A, z, s - j)[0] : 0.0;
-  double alpha[KMAX + 1];
-  bdf_alpha(kk, tau, h, alpha);
+  step_alpha<NT> alpha;
+  adj_alpha(t, A, z, s, kk, h, alpha);
   const int o = (s - Zs.lo) * n;
   vsync(t);
   if (A.tape.stride == 1) {
@@ -269,44 +284,7 @@ NB_HD inline bool adj_step(const NT& t, AdjZone& Zs, WT& w, const AT& a, const A
   int sj[KMAX + 1];
 #pragma unroll
   for (int j = 1; j <= KMAX; ++j) sj[j] = ring(s + HMAX - j);
-  for (int q = 0; q < K; ++q) {
-    const int lo = (sl * K + q) * n;
-    const double es = a.ee[sl * K + q];
-    const double ce = es * h * ia0;
-    for (int i = vbeg(t); i < n; i += vstep(t)) {
-      double v = a.lam[lo + i];
-      if (t.hasE) v = fma(ce, a.de[i], v);
-      a.mu[i] = v;
-      a.lam[lo + i] = 0.0;
-    }
-    vsync(t);
-    if (vlead(t)) a.ee[sl * K + q] = 0.0;
-    solve_MT_of(t, w.lu, a.mu);
-    vsync(t);
-#pragma unroll
-    for (int j = 1; j <= KMAX; ++j) {
-      if (j > kk) continue;
-      const int lj = (sj[j] * K + q) * n;
-      const double ma = -alpha[j];
-      for (int i = vbeg(t); i < n; i += vstep(t)) a.lam[lj + i] = fma(ma, a.mu[i], a.lam[lj + i]);
-      if (t.hasE && vlead(t)) a.ee[sj[j] * K + q] = fma(-es * ia0, alpha[j], a.ee[sj[j] * K + q]);
-    }
-    const double muT = t.sh ? a.mu[N] * icv : 0.0;
-    double gt = 0.0;
-    for (int r = vbeg(t); r < t.R; r += vstep(t)) {
-      double acc = 0.0;
-      for (int e = g.rg_ptr[r]; e < g.rg_ptr[r + 1]; ++e)
-        acc = fma(g.rg_c[e], a.mu[g.rg_i[e]], acc);
-      const double Qr = g.Q[r];
-      acc = fma(muT, Qr, acc);
-      const double v = w.rr[r] * fma(h, acc, ce * Qr);
-      a.gr[q * t.R + r] += v;
-      if (!t.sh) gt = fma(v, w.g[r], gt);
-    }
-    gt = vsum(t, gt);
-    if (vlead(t)) a.gt[q] += gt;
-    vsync(t);
-  }
+  adj_sets(t, w, a, K, kk, sl, sj, alpha, h, ia0, icv);
   Zs.s = s - 1;
   if (Zs.s == 0) return true;
   if (Zs.s < Zs.lo) seg_start(t, Zs, w, A, Zs.s);

@@ -109,6 +109,37 @@ struct BlobHeader {
   int32_t o_dej_ptr;    // int32 [n+1] derivative terms taken by species j
   int32_t o_dej_d;      // int16 [nd] those terms, in increasing order
   int32_t n_lrow, pad3_;
+  // programs of a team of threads that owns one zone (coop.cuh), all in
+  // position (elimination) order.  A column program's entry is slot |
+  // (2 row + parity) << 16: column k's update of `row`; parity is that of the
+  // entry's place in its row, which picks the partial sum it adds to in the
+  // lane kernel's order.
+  int32_t o_cl, o_cl_ptr;     // L by columns      uint32, int32 [n+1]
+  int32_t o_cu, o_cu_ptr;     // U by columns
+  int32_t o_cut, o_cut_ptr;   // U^T by columns (rows of U)
+  int32_t o_clt, o_clt_ptr;   // L^T by columns (rows of L)
+  // row programs of the back substitutions, rows grouped by dependency level:
+  // entries slot | col << 16 in increasing col
+  int32_t o_ru, o_ru_ptr;     // rows of U; entries of row k in [ptr[k], ptr[k+1])
+  int32_t o_ru_tail;          // int32 [tail] first entry of row k in the dense block's columns
+  int32_t o_ru_row, o_ru_lev; // int16 [n] rows by level, int16 [n_ru_lev + 1]
+  int32_t o_rlt, o_rlt_ptr;   // rows of L^T
+  int32_t o_rlt_row, o_rlt_lev;
+  int32_t n_ru_lev, n_rlt_lev;
+  int32_t o_pos;              // int16 [n] position of original index i
+  int32_t o_dpos;             // int16 [n] slot of the diagonal at position k
+  // gathers by length: the first *_split entries are long (each by two
+  // threads, one partial sum each), the rest go one per thread; Jacobian
+  // slots from js_fill on gather nothing
+  int32_t o_js_ord, js_split, js_fill;   // int16 [nnz] slots
+  int32_t o_rhs_ord, rhs_split;          // int16 [N] species
+  // the trailing dense block: position of its first pivot, its first slot;
+  // entry (i, j) is slot tail_slot + (i - tail) (n - tail) + j - tail
+  int32_t tail, tail_slot;
+  // a team's arrays, in doubles: thot of them kept close (shared memory),
+  // then f0 and the history
+  int32_t th_x, th_xp, th_psi, th_iw, th_tmp, th_pv, th_k, th_g, th_rr, th_kp, th_lu, th_y, th_f,
+      th_dt, th_eh, th_th, thot, tc_g, tc_kp, tc_f0, tc_xh, tcold;
 };
 
 }  // namespace nb

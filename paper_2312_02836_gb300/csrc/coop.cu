@@ -1,0 +1,169 @@
+// coop.cu -- the persistent kernels that give a zone to a team of threads
+// (coop.cuh), and their launches.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "blob.h"
+#include "coop.cuh"
+#include "host.h"
+#include "../../include/netburn.h"
+
+using namespace nb;
+
+namespace {
+
+// One zone per team of P threads (coop.cuh), sums of pattern S.  MEM 0: the
+// team's arrays in the global workspace; 1: its Newton-loop arrays in shared
+// memory, f0 and the history in the workspace.  B.smem_warps holds the doubles
+// between one team's arrays and the next in shared memory.
+template <int P, int S, int MEM, int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, MINB) k_burn_coop(const __grid_constant__ BurnParams B, const __grid_constant__ BlobHeader H) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const unsigned char* blob = B.blob;
+  if (B.blob_in_smem) {
+    const int4* src = reinterpret_cast<const int4*>(B.blob);
+    int4* dst = reinterpret_cast<int4*>(sm);
+    for (int i = threadIdx.x; i < B.blob_bytes / 16; i += blockDim.x) dst[i] = src[i];
+    __syncthreads();
+    blob = sm;
+  }
+  unsigned char* rest = sm + (B.blob_in_smem ? B.blob_bytes : 0);
+  const TNet<P, S> t(BlobDims(blob, H), reinterpret_cast<unsigned long long*>(rest));
+  double* smd = reinterpret_cast<double*>(rest + team_scratch_bytes(P));
+  const int tib = threadIdx.x / P;
+  const long long team = (long long)blockIdx.x * (blockDim.x / P) + tib;
+  const int thot = H.thot, tcold = H.tcold;
+  CWS w;
+  if constexpr (MEM == 1) {
+    w = make_cws(H, smd + (size_t)tib * B.smem_warps, B.ws + team * tcold);
+  } else {
+    double* hot = B.ws + team * (thot + tcold);
+    w = make_cws(H, hot, hot + thot);
+  }
+  coop_claim_loop(t, w, B);
+}
+
+// One built form of the kernel.
+struct TeamKernel {
+  int P, S, mem;
+  void (*fn)(const BurnParams, const BlobHeader);
+};
+#define NB_TEAM(P, S, MEM, TPB, MINB) {P, S, MEM, k_burn_coop<P, S, MEM, TPB, MINB>}
+// All take the registers they want (254): a 168-register form for three
+// blocks of four warps per SM, which the earlier kernel gained from, spills
+// and ran 1030 ms where this one, with two blocks, takes 936 ms (48 species,
+// 65,536 zones).
+const TeamKernel kTeamKernels[] = {
+    NB_TEAM(32, 32, 0, 256, 1),   NB_TEAM(32, 32, 1, 256, 1),   NB_TEAM(64, 32, 1, 64, 4),
+    NB_TEAM(128, 32, 1, 128, 2),  NB_TEAM(64, 64, 0, 64, 1),    NB_TEAM(64, 64, 1, 64, 1),
+    NB_TEAM(256, 64, 1, 256, 1),  NB_TEAM(128, 128, 0, 128, 1), NB_TEAM(128, 128, 1, 128, 1),
+    NB_TEAM(256, 128, 1, 256, 1),
+};
+#undef NB_TEAM
+
+const TeamKernel& team_kernel(int P, int S, int mem) {
+  const TeamKernel* hit = kTeamKernels;
+  for (const TeamKernel& k : kTeamKernels)
+    if (k.P == P && k.S == S && k.mem == mem) hit = &k;
+  return *hit;
+}
+
+// Launch kernel k with `threads` per block (a multiple of its P), at most
+// `bps` blocks per SM (0: as many as fit).
+int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel& k, int threads,
+                int bps, int in_smem, cudaStream_t st) {
+  const int teams = threads / k.P;
+  const size_t blob_b = in_smem ? (size_t)net->h.bytes : 0;
+  const int stride = k.mem == 0 ? 0 : net->h.thot;
+  const size_t dyn = blob_b + team_scratch_bytes(k.P) + (size_t)teams * stride * sizeof(double);
+  if (dyn > net->smem_optin) return NB_E_TOO_LARGE;
+  CK(cudaFuncSetAttribute((const void*)k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  int occ = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k.fn, threads, dyn));
+  if (occ < 1) return NB_E_TOO_LARGE;
+  long long blocks = (long long)std::max(1, std::min(bps > 0 ? bps : occ, occ)) * net->sm_count;
+  blocks = std::min(blocks, (P.Z + teams - 1) / teams);
+  const size_t per_team =
+      8 * ((size_t)(k.mem == 0 ? net->h.thot : 0) + net->h.tcold);
+  size_t need = std::max<size_t>((size_t)blocks * teams * per_team, 256);
+  // the pre-pass runs one zone per lane: enough lanes for every SM (one block
+  // of 128 for all zones took 0.9 s for 262,144 zones of the 48-species
+  // network), at most 64 an SM, since a lane's arrays hold 25 to 120 KB
+  const long long elanes =
+      std::min<long long>((P.Z + 127) / 128 * 128, ((long long)net->sm_count * 64 + 127) / 128 * 128);
+  if (o.schedule == 1)
+    need = std::max(need, (size_t)elanes * (size_t)net->h.lane_doubles * sizeof(double));
+  int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);
+  if (rc) return rc;
+  P.ws = net->ws;
+  P.queue = net->queue;
+  P.blob_in_smem = in_smem;
+  P.smem_warps = stride;
+  P.order = nullptr;
+  if (o.schedule == 1 && P.Z > 1) {
+    rc = nb::schedule_longest_first(net, P, elanes, st);
+    if (rc) return rc;
+  }
+  CK(cudaMemsetAsync(net->queue, 0, sizeof(unsigned long long), st));
+  k.fn<<<(unsigned)blocks, threads, dyn, st>>>(P, net->h);
+  CK(cudaGetLastError());
+  return NB_OK;
+}
+
+}  // namespace
+
+// Sums in team order of S = 32 x warps_per_zone partial sums.
+// threads_per_block (default: the warps whose Newton-loop arrays fit in
+// shared memory, at most 4 of them) and blocks_per_sm bound the zones in
+// flight; ws_in_shared 0 keeps all arrays in global memory, otherwise
+// (default) in shared memory when they fit; blob_in_shared as for the
+// persistent kernel.  The threads P of a team follow the work and the zones:
+//  * a large network (1,000 and more update pairs a pivot, 128 species:
+//    1,763) keeps eight warps busy whatever the number of zones: 300 zones
+//    take 492 ms with two warps, 296 ms with eight (128 species, S = 64);
+//    one warp and four (S = 32): 247 and 123 ms.  Two teams of eight warps
+//    don't fit an SM's registers, so with S = 32, for which a zone has one
+//    of several warps of a block's, it is four;
+//  * else (48 species: 238 pairs) one warp a zone does the most zones per
+//    second (16,384 zones 237 ms, two warps 560 ms), but with few zones per
+//    SM the longest zone sets the time, and two or four warps shorten it:
+//    16 zones 100, 84, 77 ms with 1, 2, 4 warps; 912 zones 100, 84, 82 ms;
+//    2,048 zones 108, 83, 83 ms; 4,096 zones 110, 167, 168 ms.
+int nb::launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st) {
+  const size_t blob_b = (size_t)net->h.bytes;
+  const size_t hot_team = (size_t)net->h.thot * sizeof(double);
+  const int wpz = o.warps_per_zone <= 1 ? 1 : o.warps_per_zone;
+  if (o.warps_per_zone < 0 || (wpz != 1 && wpz != 2 && wpz != 4)) return NB_E_ARG;
+  if (wpz == 1 && o.threads_per_block > 0 &&
+      (o.threads_per_block % 32 != 0 || o.threads_per_block > 256))
+    return NB_E_ARG;
+  const size_t scratch = team_scratch_bytes(64);
+  const bool hot_smem = o.ws_in_shared != 0 && hot_team + scratch <= net->smem_optin;
+  int in_smem = o.blob_in_shared;
+  if (in_smem < 0)
+    in_smem = blob_b <= 96 * 1024 && blob_b + (hot_smem ? hot_team : 0) + scratch <= net->smem_optin;
+  const size_t fixed = (in_smem ? blob_b : 0) + scratch;
+  const int S = 32 * wpz;
+  // an explicit block of several zones has to fit with one zone per warp
+  const size_t warp_b = (size_t)net->h.hot_doubles * sizeof(double);
+  const int warps_asked = wpz == 1 ? o.threads_per_block / 32 : 0;
+  if (warps_asked > 0 && o.ws_in_shared != 0 && warp_b <= net->smem_optin &&
+      (in_smem ? blob_b : 0) + warps_asked * warp_b > net->smem_optin)
+    return NB_E_TOO_LARGE;
+  const bool large = net->h.nD >= 1024 * net->h.n;
+  int T = S;
+  if (hot_smem) {
+    if (large) T = wpz == 1 ? 128 : 256;
+    else if (wpz == 1) T = P.Z <= 6LL * net->sm_count ? 128 : P.Z <= 16LL * net->sm_count ? 64 : 32;
+  }
+  int threads = T;
+  if (T == 32) {
+    int warps = warps_asked > 0 ? warps_asked : 4;
+    if (hot_smem)
+      while (warps > 1 && fixed + (size_t)warps * hot_team > net->smem_optin) --warps;
+    threads = 32 * warps;
+  }
+  return launch_team(net, P, o, team_kernel(T, S, hot_smem ? 1 : 0), threads, o.blocks_per_sm,
+                     in_smem, st);
+}

@@ -149,8 +149,10 @@ NB_HD __forceinline__ WS make_ws(const Net& t, double* lane_base) {
 // ---------------------------------------------------------------- model
 
 // k_r of reaction r (and g_r = d ln lambda_r / dT9 when g) at T9 with powers p
-// (tc: the temperature cell of the rate tables at T9)
-NB_HD __forceinline__ double rate_full(const Net& t, const Zone& s, int r, const TPow& p,
+// (tc: the temperature cell of the rate tables at T9); NET: Net or another
+// view of the same rate arrays
+template <class NET>
+NB_HD __forceinline__ double rate_full(const NET& t, const Zone& s, int r, const TPow& p,
                                        double T9, const TCell& tc, double* g) {
   const double* a = t.coef + 7 * r;
   const int tb = t.tab_of ? t.tab_of[r] : -1;

@@ -87,4 +87,11 @@ inline int ensure(void** p, size_t* have, size_t need) {
   *have = need;
   return NB_OK;
 }
+
+// Longest-first claim order: h0 of every zone (a pre-pass on `lanes` lanes of
+// the workspace already allocated), then a radix sort of (h0, zone).  Sets
+// P.order.  (burn.cu)
+int schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaStream_t st);
+// The cooperative launch (coop.cu).  Caller holds net->mu.
+int launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st);
 }  // namespace nb

@@ -70,10 +70,18 @@ template <class NT>
 NB_HD __forceinline__ constexpr int vstep(const NT&) {
   if constexpr (is_coop<NT>::value) return NT::width; else return 1;
 }
-// sum over the zone's threads of their partial sums (the same bits in all)
-template <class NT>
-NB_HD __forceinline__ double vsum(const NT& t, double x) {
-  if constexpr (is_coop<NT>::value) return t.sum(x); else return x;
+// sum_{i<cnt} f(i): acc <- f(i, acc) in the network type's own order (one
+// chain in index order for one zone per lane)
+template <class NT, class F>
+NB_HD __forceinline__ double vsum1(const NT& t, int cnt, F f) {
+  if constexpr (is_coop<NT>::value) {
+    return t.sum1(cnt, f);
+  } else {
+    double acc = 0.0;
+    NB_UNROLL
+    for (int i = 0; i < cnt; ++i) acc = f(i, acc);
+    return acc;
+  }
 }
 template <class NT>
 NB_HD __forceinline__ bool vall(const NT& t, bool b) {
@@ -88,6 +96,33 @@ NB_HD __forceinline__ void vsync(const NT& t) {
 template <class NT>
 NB_HD __forceinline__ bool vlead(const NT& t) {
   if constexpr (is_coop<NT>::value) return t.lane == 0; else return true;
+}
+
+// Network types whose warps of a block run the step's phases together (the
+// generated kernel: its straight-line code is larger than the instruction
+// caches, and a block's warps share what they fetch only while they are in
+// the same part of it)
+template <class NT, class = void>
+struct in_step {
+  static constexpr bool value = false;
+};
+template <class NT>
+struct in_step<NT, decltype((void)NT::in_step)> {
+  static constexpr bool value = NT::in_step;
+};
+template <class NT>
+NB_HD __forceinline__ void phase_sync(const NT&) {
+#ifdef __CUDA_ARCH__
+  if constexpr (in_step<NT>::value) __syncthreads();
+#endif
+}
+// does this thread (with phases in step: any thread of the block) go on?
+template <class NT>
+NB_HD __forceinline__ bool phase_any(const NT&, bool go) {
+#ifdef __CUDA_ARCH__
+  if constexpr (in_step<NT>::value) return __syncthreads_or(go) != 0;
+#endif
+  return go;
 }
 
 // lane-strided view of one per-lane array
@@ -438,9 +473,7 @@ NB_HD __forceinline__ double rate_near(double kref, double de) {
 template <class NT, class V>
 NB_HD __forceinline__ double heat_capacity(const NT& t, const V& v) {
   if constexpr (is_coop<NT>::value) {
-    double sy = 0.0;
-    for (int i = vbeg(t); i < t.N; i += vstep(t)) sy += v[i];
-    sy = vsum(t, sy);
+    const double sy = t.sum2(t.N, [&](int i, double a) { return a + v[i]; });
     const double T9 = v[t.N];
     return 1.5 * sy + 1e-3 * T9 * T9 * T9;
   }
@@ -478,14 +511,6 @@ NB_HD __forceinline__ TRow t_row(double ed, double cv, double T9) {
 // compare squares, which spares a square root per norm)
 template <class NT, class WT, class V>
 NB_HD __forceinline__ double wnorm2(const NT& t, const WT& w, const V& v) {
-  if constexpr (is_coop<NT>::value) {
-    double sq = 0.0;
-    for (int i = vbeg(t); i < t.n; i += vstep(t)) {
-      const double q = v[i] * w.iw[i];
-      sq = fma(q, q, sq);
-    }
-    return vsum(t, sq) * t.inv_n;
-  }
   double s0 = 0.0, s1 = 0.0;
   int i = 0;
   NB_UNROLL
@@ -524,7 +549,7 @@ NB_HD __forceinline__ void hist_combine(const NT& t, const WT& w, int cnt, const
   NB_UNROLL
   for (int i = 0; i < NT::n; ++i) out[i] = acc[i];
 #else
-  for (int i = vbeg(t); i < t.n; i += vstep(t)) {
+  for (int i = 0; i < t.n; ++i) {
     double acc = 0.0;
     for (int j = 0; j < cnt; ++j) acc = fma(c[j], w.xh[base[j] + i], acc);
     out[i] = acc;
@@ -590,12 +615,23 @@ NB_HD __forceinline__ double order_estimate(const NT& t, const Zone& s, WT& w, i
   const int b0 = hslot(s, 0) * t.n;
   double acc = 0.0;
   NB_UNROLL
-  for (int i = vbeg(t); i < t.n; i += vstep(t)) {
+  for (int i = 0; i < t.n; ++i) {
     const double v = c * (w.xh[b0 + i] - w.tmp[i]) * w.iw[i];
     acc = fma(v, v, acc);
   }
-  return vsum(t, acc) * t.inv_n;   // E_q^2
+  return acc * t.inv_n;   // E_q^2
 }
+
+// The pieces of a step attempt that a network type may do its own way: a
+// team of threads overloads them (coop.cuh).
+
+// alpha_0..alpha_KMAX of one step
+template <class NT>
+struct step_alpha {
+  double a[KMAX + 1];
+  NB_HD __forceinline__ double& operator[](int j) { return a[j]; }
+  NB_HD __forceinline__ double operator[](int j) const { return a[j]; }
+};
 
 // Record an accepted point (time, step, order; state and energy when the
 // record is a kept one); false when the zone's tape is full.
@@ -645,6 +681,79 @@ NB_HD __forceinline__ void bdf_alpha(int kk, const double* tau, double h, double
 #pragma unroll
   for (int j = 1; j <= KMAX; ++j)
     if (j > kk) alpha[j] = 0.0;
+}
+
+// alpha_j of the step from the history to t_new, psi = sum_{j>=1} alpha_j
+// x_{n+1-j}, and the error weights from x_n
+template <class NT, class WT>
+NB_HD __forceinline__ void step_coeffs(const NT& t, const Zone& s, WT& w, double atol, double rtol,
+                                       double h, double t_new, int kk, step_alpha<NT>& alpha) {
+  const int n = t.n;
+  // alpha_j = h l_j'(t_new) over t_new, t_n, .., t_{n+1-kk}
+  double tau[KMAX + 1];
+  tau[0] = t_new;
+#pragma unroll 1
+  for (int j = 1; j <= kk; ++j) tau[j] = w.th[hslot(s, j - 1)];
+  bdf_alpha(kk, tau, h, alpha.a);
+  int base[KMAX];
+#pragma unroll 1
+  for (int j = 0; j < kk; ++j) base[j] = hslot(s, j) * n;
+  hist_combine(t, w, kk, alpha.a + 1, base, w.psi);
+  const int b0 = hslot(s, 0) * n;
+  NB_UNROLL
+  for (int i = 0; i < n; ++i) w.iw[i] = recip1(atol + rtol * fabs(w.xh[b0 + i]));
+}
+
+// the degree-q predictor at t_new through history 0..q
+template <class NT, class WT>
+NB_HD __forceinline__ void predict(const NT& t, const Zone& s, WT& w, int q, double t_new) {
+  extrapolate(t, s, w, 0, q, t_new, w.xp);
+}
+
+// one modified-Newton correction: d = -(alpha0 x + psi - h f), M d' = d,
+// x += d'; returns ||d'||^2
+template <class NT, class WT>
+NB_HD __forceinline__ double newton_correct(const NT& t, WT& w, double alpha0, double h) {
+  NB_UNROLL
+  for (int i = 0; i < t.n; ++i) w.d[i] = -(fma(alpha0, w.x[i], w.psi[i]) - h * w.f[i]);
+  solve_M(t, w, w.d);
+  NB_UNROLL
+  for (int i = 0; i < t.n; ++i) w.x[i] += w.d[i];
+  return wnorm2(t, w, w.d);
+}
+
+// err^2 = ||c (x - xp)||^2
+template <class NT, class WT>
+NB_HD __forceinline__ double error_norm2(const NT& t, WT& w, double c) {
+  double acc = 0.0;
+  NB_UNROLL
+  for (int i = 0; i < t.n; ++i) {
+    const double v = c * (w.x[i] - w.xp[i]) * w.iw[i];
+    acc = fma(v, v, acc);
+  }
+  return acc * t.inv_n;
+}
+
+// Step-size factor after an accepted step at order k whose estimate was
+// err2, with the best of orders k-1, k, k+1 (best_q); (k+1 only with k+3
+// points held)
+template <class NT, class WT>
+NB_HD __forceinline__ double order_factor(const NT& t, const Zone& s, WT& w, double err2,
+                                          double h, int& best_q) {
+  const int k = s.k;
+  best_q = k;
+  // E_k is the step's own error estimate: the same extrapolation through
+  // the same points at the same time, so the same bits
+  double best = step_factor(err2, k);
+  if (k > 1) {
+    const double fq = step_factor(order_estimate(t, s, w, k - 1, h), k - 1);
+    if (fq > best) { best = fq; best_q = k - 1; }
+  }
+  if (k < KMAX && s.nh >= k + 3) {
+    const double fq = step_factor(order_estimate(t, s, w, k + 1, h), k + 1);
+    if (fq > best) { best = fq; best_q = k + 1; }
+  }
+  return best;
 }
 
 // ---------------------------------------------------------------- zone start
@@ -700,17 +809,17 @@ NB_HD __forceinline__ bool zone_init(const NT& t, Zone& s, WT& w, const BurnPara
   if (!fin) { s.status = NB_Z_NONFINITE; return true; }
   if (!(s.tend > 0.0)) return true;
   // starting step: Hairer-Norsett-Wanner I, Sec. II.4, p = 1
-  double s0 = 0.0, s1 = 0.0;
   NB_UNROLL
-  for (int i = vbeg(t); i < n; i += vstep(t)) {
-    const double iw = recip1(P.atol + P.rtol * fabs(x0[i]));
-    w.iw[i] = iw;
-    const double a = x0[i] * iw, b = w.f0[i] * iw;
-    s0 = fma(a, a, s0);
-    s1 = fma(b, b, s1);
-  }
-  s0 = vsum(t, s0);
-  s1 = vsum(t, s1);
+  for (int i = vbeg(t); i < n; i += vstep(t)) w.iw[i] = recip1(P.atol + P.rtol * fabs(x0[i]));
+  vsync(t);
+  const double s0 = vsum1(t, n, [&](int i, double acc) {
+    const double a = x0[i] * w.iw[i];
+    return fma(a, a, acc);
+  });
+  const double s1 = vsum1(t, n, [&](int i, double acc) {
+    const double b = w.f0[i] * w.iw[i];
+    return fma(b, b, acc);
+  });
   const double d0 = sqrt(s0 / n), d1 = sqrt(s1 / n);
   double hp = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
   if (hp > s.tend) hp = s.tend;
@@ -725,14 +834,12 @@ NB_HD __forceinline__ bool zone_init(const NT& t, Zone& s, WT& w, const BurnPara
   eval_terms(t, w, w.x);
   eval_f(t, w, w.x, w.f);
   s.c_rhs++;
-  double s2 = 0.0;
   const double ihp = 1.0 / hp;
-  NB_UNROLL
-  for (int i = vbeg(t); i < n; i += vstep(t)) {
+  vsync(t);
+  const double s2 = vsum1(t, n, [&](int i, double acc) {
     const double q = (w.f[i] - w.f0[i]) * ihp * w.iw[i];
-    s2 = fma(q, q, s2);
-  }
-  s2 = vsum(t, s2);
+    return fma(q, q, acc);
+  });
   const double d2 = sqrt(s2 / n);
   const double dm = fmax(d1, d2);
   const double h1 = dm <= 1e-15 ? fmax(1e-6, hp * 1e-3) : sqrt(0.01 / dm);
@@ -745,201 +852,208 @@ NB_HD __forceinline__ bool zone_init(const NT& t, Zone& s, WT& w, const BurnPara
 
 // ---------------------------------------------------------------- one attempt
 
+// What an attempt found: Newton converged, the LU was sound; of a converged
+// full attempt the error norm, and of an acceptable one edot at the solution.
+struct Attempt {
+  bool converged, lu_ok;
+  double err2, ed;
+};
+
 // The computation of one step attempt from t_n = s.t to t_new with step h at
 // order kk: BDF coefficients, history sum, weights from x_n, predictor,
-// Jacobian and LU at the predictor, modified Newton.  Leaves the solution in
-// w.x and the predictor in w.xp, alpha_0..alpha_kk in alpha and, with
-// self-heating, the reference temperature of the rates in Tref (powers
-// pref); returns true when Newton converged.  The forward burn and the
+// Jacobian and LU at the predictor, modified Newton; FULL: the error norm
+// and, when it accepts, the energy rate.  Leaves the solution in w.x, the
+// predictor in w.xp and alpha_0..alpha_kk in alpha.  The forward burn and the
 // adjoint's recomputation of checkpointed segments both run it, so that they
-// produce the same bits.
-template <class NT, class WT>
-NB_HD __forceinline__ bool attempt_solve(const NT& t, Zone& s, WT& w, double atol, double rtol,
-                                         double h, double t_new, int kk, double* alpha,
-                                         TPow& pref, double& Tref, bool& lu_ok) {
+// produce the same bits.  Threads without an attempt pass run = false and
+// only keep the phases of their block.
+template <bool FULL, class NT, class WT>
+NB_HD __forceinline__ Attempt attempt_solve(const NT& t, Zone& s, WT& w, bool run, double atol,
+                                            double rtol, double h, double t_new, int kk,
+                                            step_alpha<NT>& alpha) {
   const int n = t.n, N = t.N;
-  vsync(t);   // the history written by the last accepted step
-  // alpha_j = h l_j'(t_new) over t_new, t_n, .., t_{n+1-kk}
-  double tau[KMAX + 1];
-  tau[0] = t_new;
-#pragma unroll 1
-  for (int j = 1; j <= kk; ++j) tau[j] = w.th[hslot(s, j - 1)];
-  bdf_alpha(kk, tau, h, alpha);
-  // psi = sum_{j>=1} alpha_j x_{n+1-j}; weights from x_n
-  {
-    int base[KMAX];
-#pragma unroll 1
-    for (int j = 0; j < kk; ++j) base[j] = hslot(s, j) * n;
-    hist_combine(t, w, kk, alpha + 1, base, w.psi);
-    const int b0 = hslot(s, 0) * n;
+  Attempt at{false, false, 0.0, 0.0};
+  if (run) {
+    vsync(t);   // the history written by the last accepted step
+    step_coeffs(t, s, w, atol, rtol, h, t_new, kk, alpha);
+    // predictor
+    if (s.nh >= kk + 1) predict(t, s, w, kk, t_new);
+    else if (s.nh >= 2) predict(t, s, w, s.nh - 1, t_new);
+    else {
+      const int b0 = hslot(s, 0) * n;
+      NB_UNROLL
+      for (int i = vbeg(t); i < n; i += vstep(t)) w.xp[i] = fma(h, w.f0[i], w.xh[b0 + i]);
+    }
     NB_UNROLL
-    for (int i = vbeg(t); i < n; i += vstep(t))
-      w.iw[i] = recip1(atol + rtol * fabs(w.xh[b0 + i]));
+    for (int i = vbeg(t); i < n; i += vstep(t)) w.x[i] = w.xp[i];
+    vsync(t);
   }
-  // predictor
-  if (s.nh >= kk + 1) extrapolate(t, s, w, 0, kk, t_new, w.xp);
-  else if (s.nh >= 2) extrapolate(t, s, w, 0, s.nh - 1, t_new, w.xp);
-  else {
-    const int b0 = hslot(s, 0) * n;
-    NB_UNROLL
-    for (int i = vbeg(t); i < n; i += vstep(t)) w.xp[i] = fma(h, w.f0[i], w.xh[b0 + i]);
-  }
-  NB_UNROLL
-  for (int i = vbeg(t); i < n; i += vstep(t)) w.x[i] = w.xp[i];
-  vsync(t);
+  phase_sync(t);
   // Jacobian at the predictor, M, LU; with self-heating the predictor's
   // temperature is the attempt's reference for the rates
-  Tref = 0.0;
-  if (t.sh) {
-    Tref = w.x[N];
-    pref = t_powers(Tref, true, s.scr);
-    eval_rates(t, s, w, pref, Tref, true);
-    save_ref_rates(t, w);
-    s.c_teval++;
+  double Tref = 0.0;
+  TPow pref;
+  if (run) {
+    if (t.sh) {
+      Tref = w.x[N];
+      pref = t_powers(Tref, true, s.scr);
+      eval_rates(t, s, w, pref, Tref, true);
+      save_ref_rates(t, w);
+      s.c_teval++;
+    }
+    eval_terms(t, w, w.x);
   }
-  eval_terms(t, w, w.x);
-  assemble_M(t, w, w.x, alpha[0], h);
-  s.c_jac++;
-  bool ok = factor_M(t, w);
-  lu_ok = ok;
-  // modified Newton
-  bool converged = false;
+  phase_sync(t);
+  if (run) {
+    assemble_M(t, w, w.x, alpha[0], h);
+    s.c_jac++;
+    at.lu_ok = factor_M(t, w);
+  }
+  // modified Newton; a pass after convergence evaluates the rates and terms
+  // of the solution for the energy, from the one place in the code that does
+  bool go = run && at.lu_ok, energy = false;
   double nrm_prev = 0.0;
-  for (int m = 0; ok && m < 4; ++m) {
+  for (int m = 0; phase_any(t, go); ++m) {
+    if (!go) continue;
     if (m > 0) {
       if (t.sh) { eval_rates_near(t, s, w, w.x[N], pref, Tref); s.c_teval++; }
       eval_terms(t, w, w.x);
     }
+    if (energy) {
+      at.ed = eval_edot(t, w);
+      s.c_edot++;
+      go = false;
+      continue;
+    }
     eval_f(t, w, w.x, w.f);
     s.c_rhs++;
-    NB_UNROLL
-    for (int i = vbeg(t); i < n; i += vstep(t))
-      w.d[i] = -(fma(alpha[0], w.x[i], w.psi[i]) - h * w.f[i]);
-    solve_M(t, w, w.d);
-    NB_UNROLL
-    for (int i = vbeg(t); i < n; i += vstep(t)) w.x[i] += w.d[i];
-    vsync(t);
+    const double nrm2 = newton_correct(t, w, alpha[0], h);
     s.c_newton++;
-    const double nrm2 = wnorm2(t, w, w.d);
-    if (!finite_bits(nrm2)) { ok = false; break; }
-    if (nrm2 <= 1e-6) { converged = true; break; }          // ||d|| <= 1e-3
-    if (m > 0) {
-      if (nrm2 > 0.81 * nrm_prev) { ok = false; break; }     // theta > 0.9
-      const double theta = sqrt(nrm2 / nrm_prev);
-      if (theta / (1.0 - theta) * sqrt(nrm2) <= 1e-3) { converged = true; break; }
+    if (!finite_bits(nrm2)) {
+      go = false;
+    } else if (nrm2 <= 1e-6) {                       // ||d|| <= 1e-3
+      at.converged = true;
+    } else if (m > 0) {
+      if (nrm2 > 0.81 * nrm_prev) {                  // theta > 0.9
+        go = false;
+      } else {
+        const double theta = sqrt(nrm2 / nrm_prev);
+        at.converged = theta / (1.0 - theta) * sqrt(nrm2) <= 1e-3;
+      }
     }
     nrm_prev = nrm2;
+    if (at.converged) {
+      if constexpr (FULL) {
+        // local error estimate
+        const double c = s.nh >= kk + 1 ? h / (t_new - w.th[hslot(s, kk)]) : 0.5;
+        at.err2 = error_norm2(t, w, c);
+        energy = at.err2 <= 1.0 && t.hasE;
+      }
+      go = energy;
+    } else if (m == 3) {
+      go = false;
+    }
   }
-  return converged;
+  return at;
 }
 
-// One step attempt.  Returns true when the zone is finished.
+// The factor on h after an accepted step: when the zone may change its order
+// (sel), the best of orders k-1, k, k+1, else that of the step's own order kk.
 template <class NT, class WT>
-NB_HD __forceinline__ bool zone_attempt(const NT& t, Zone& s, WT& w, const BurnParams& P) {
-  const int n = t.n, N = t.N;
-  if (s.c_acc + s.c_rej_err + s.c_rej_newton >= P.max_attempts) {
-    s.status = NB_Z_MAX_STEPS;
-    return true;
-  }
+NB_HD __forceinline__ double next_factor(const NT& t, const Zone& s, WT& w, bool acc, bool sel,
+                                         double err2, double h, int kk, int& best_q) {
+  best_q = s.k;
+  if (!acc) return 1.0;
+  return sel ? order_factor(t, s, w, err2, h, best_q) : step_factor(err2, kk);
+}
+
+// One step attempt of a thread with run set.  Returns true when its zone is
+// finished.
+template <class NT, class WT>
+NB_HD __forceinline__ bool zone_attempt(const NT& t, Zone& s, WT& w, const BurnParams& P,
+                                        bool run = true) {
+  const int n = t.n;
+  bool done = false;
   double h = s.h;
-  if (h < 1e-30 * s.tend || h < 1e-14 * s.t) {
+  if (run && s.c_acc + s.c_rej_err + s.c_rej_newton >= P.max_attempts) {
+    s.status = NB_Z_MAX_STEPS;
+    done = true;
+  } else if (run && (h < 1e-30 * s.tend || h < 1e-14 * s.t)) {
     s.status = NB_Z_DT_UNDERFLOW;
-    return true;
+    done = true;
   }
+  run = run && !done;
   double t_new;
   if (s.t + h >= s.tend) { h = s.tend - s.t; t_new = s.tend; }
   else t_new = s.t + h;
   const int kk = s.k < s.nh ? s.k : s.nh;
-  double alpha[KMAX + 1];
-  TPow pref;
-  double Tref;
-  bool lu_ok;
-  const bool converged =
-      attempt_solve(t, s, w, P.atol, P.rtol, h, t_new, kk, alpha, pref, Tref, lu_ok);
-  if (!converged) {
+  step_alpha<NT> alpha;
+  const Attempt at = attempt_solve<true>(t, s, w, run, P.atol, P.rtol, h, t_new, kk, alpha);
+  bool acc = false;
+  if (run && !at.converged) {
     s.c_rej_newton++;
-    if (++s.nfail >= 10) { s.status = lu_ok ? NB_Z_NEWTON_FAIL : NB_Z_SINGULAR; return true; }
-    s.h = h * 0.25;
-    return false;
-  }
-  s.nfail = 0;
-  // local error estimate
-  const double c = s.nh >= kk + 1 ? h / (t_new - w.th[hslot(s, kk)]) : 0.5;
-  double err2;   // err^2
-  {
-    double acc = 0.0;
-    NB_UNROLL
-    for (int i = vbeg(t); i < n; i += vstep(t)) {
-      const double v = c * (w.x[i] - w.xp[i]) * w.iw[i];
-      acc = fma(v, v, acc);
+    if (++s.nfail >= 10) {
+      s.status = at.lu_ok ? NB_Z_NEWTON_FAIL : NB_Z_SINGULAR;
+      done = true;
+    } else {
+      s.h = h * 0.25;
     }
-    err2 = vsum(t, acc) * t.inv_n;
+  } else if (run) {
+    s.nfail = 0;
+    acc = at.err2 <= 1.0;
+    if (!acc) {
+      s.c_rej_err++;
+      const double fac = finite_bits(at.err2) ? err_factor(at.err2, kk) : 0.2;
+      s.h = h * (fac > 0.2 ? fac : 0.2);
+    }
   }
-  if (!(err2 <= 1.0)) {
-    s.c_rej_err++;
-    const double fac = finite_bits(err2) ? err_factor(err2, kk) : 0.2;
-    s.h = h * (fac > 0.2 ? fac : 0.2);
-    return false;
-  }
-  // accept
-  double E_new = 0.0;
-  if (t.hasE) {
-    if (t.sh) { eval_rates_near(t, s, w, w.x[N], pref, Tref); s.c_teval++; }
-    eval_terms(t, w, w.x);
-    const double ed = eval_edot(t, w);
-    s.c_edot++;
-    double acc = 0.0;
+  if (acc) {
+    double E_new = 0.0;
+    if (t.hasE) {
+      double e = 0.0;
 #pragma unroll 1
-    for (int j = 1; j <= kk; ++j) acc = fma(alpha[j], w.eh[hslot(s, j - 1)], acc);
-    E_new = (h * ed - acc) / alpha[0];
-  }
-  // push the new point into the history ring
-  s.hh = s.hh == 0 ? HMAX - 1 : s.hh - 1;
-  vsync(t);   // every thread has read the ring's old scalars
-  {
-    const int b0 = s.hh * n;
-    NB_UNROLL
-    for (int i = vbeg(t); i < n; i += vstep(t)) w.xh[b0 + i] = w.x[i];
-    if (vlead(t)) {
-      w.th[s.hh] = t_new;
-      w.eh[s.hh] = E_new;
+      for (int j = 1; j <= kk; ++j) e = fma(alpha[j], w.eh[hslot(s, j - 1)], e);
+      E_new = (h * at.ed - e) / alpha[0];
     }
+    // push the new point into the history ring
+    s.hh = s.hh == 0 ? HMAX - 1 : s.hh - 1;
+    vsync(t);   // every thread has read the ring's old scalars
+    {
+      const int b0 = s.hh * n;
+      NB_UNROLL
+      for (int i = vbeg(t); i < n; i += vstep(t)) w.xh[b0 + i] = w.x[i];
+      if (vlead(t)) {
+        w.th[s.hh] = t_new;
+        w.eh[s.hh] = E_new;
+      }
+    }
+    vsync(t);
+    if (s.nh < HMAX) s.nh++;
+    s.t = t_new;
+    s.E = E_new;
+    s.c_acc++;
+    s.c_ordsum += kk;
+    if (!tape_record(t, P, s, w.x, h, kk)) {
+      s.status = NB_Z_TAPE_FULL;
+      done = true;
+    } else if (s.t >= s.tend) {
+      s.h = h;
+      done = true;
+    }
+    acc = !done;
   }
-  vsync(t);
-  if (s.nh < HMAX) s.nh++;
-  s.t = t_new;
-  s.E = E_new;
-  s.c_acc++;
-  s.c_ordsum += kk;
-  if (!tape_record(t, P, s, w.x, h, kk)) { s.status = NB_Z_TAPE_FULL; return true; }
-  if (s.t >= s.tend) { s.h = h; return true; }
   // next step size and order
-  s.nconsec++;
-  double factor;
-  if (s.nconsec >= s.k + 1) {
-    const int k = s.k;
-    int best_q = k;
-    // E_k is the step's own error estimate: the same extrapolation through
-    // the same points at the same time, so the same bits
-    double best = step_factor(err2, k);
-    if (k > 1) {
-      const double fq = step_factor(order_estimate(t, s, w, k - 1, h), k - 1);
-      if (fq > best) { best = fq; best_q = k - 1; }
-    }
-    if (k < KMAX && s.nh >= k + 3) {
-      const double fq = step_factor(order_estimate(t, s, w, k + 1, h), k + 1);
-      if (fq > best) { best = fq; best_q = k + 1; }
-    }
-    if (best_q != k) { s.k = best_q; s.nconsec = 0; }
-    factor = best;
-  } else {
-    factor = step_factor(err2, kk);
+  if (acc) s.nconsec++;
+  int best_q;
+  double factor = next_factor(t, s, w, acc, acc && s.nconsec >= s.k + 1, at.err2, h, kk, best_q);
+  if (acc) {
+    if (best_q != s.k) { s.k = best_q; s.nconsec = 0; }
+    if (factor < 0.2) factor = 0.2;
+    if (factor > 5.0) factor = 5.0;
+    if (factor >= 1.0 && factor < 1.2) factor = 1.0;
+    s.h = h * factor;
   }
-  if (factor < 0.2) factor = 0.2;
-  if (factor > 5.0) factor = 5.0;
-  if (factor >= 1.0 && factor < 1.2) factor = 1.0;
-  s.h = h * factor;
-  return false;
+  return done;
 }
 
 // Recompute accepted step (h, t_new, order kk) of a recorded burn from the
@@ -949,11 +1063,9 @@ NB_HD __forceinline__ bool zone_attempt(const NT& t, Zone& s, WT& w, const BurnP
 template <class NT, class WT>
 NB_HD __forceinline__ bool replay_step(const NT& t, Zone& s, WT& w, double atol, double rtol,
                                        double h, double t_new, int kk) {
-  double alpha[KMAX + 1];
-  TPow pref;
-  double Tref;
-  bool lu_ok;
-  if (!attempt_solve(t, s, w, atol, rtol, h, t_new, kk, alpha, pref, Tref, lu_ok)) return false;
+  step_alpha<NT> alpha;
+  if (!attempt_solve<false>(t, s, w, true, atol, rtol, h, t_new, kk, alpha).converged)
+    return false;
   s.hh = s.hh == 0 ? HMAX - 1 : s.hh - 1;
   vsync(t);
   const int b0 = s.hh * t.n;
@@ -1027,6 +1139,8 @@ __device__ __forceinline__ void burn_claim_loop(const NT& t, WT& w, const BurnPa
   const int lane = threadIdx.x & 31;
   Zone s;
   s.z = -1;
+  s.h = s.t = s.tend = 0.0;
+  s.k = s.nh = 1;
   bool active = false, retired = false, fresh = false;
   const unsigned long long t_start = P.budget_ns ? gpu_ns() : 0ull;
   for (;;) {
@@ -1047,29 +1161,33 @@ __device__ __forceinline__ void burn_claim_loop(const NT& t, WT& w, const BurnPa
         }
       }
     }
-    if (__all_sync(0xffffffffu, retired)) break;
-    if (active) {
-      const bool expired = P.budget_ns && gpu_ns() - t_start > P.budget_ns;
-      bool done;
-      if (expired && fresh) {
-        zone_timeout_unstarted(t, s.z, P);
-        fresh = false;
-        active = false;
-        continue;
-      }
-      if (expired) {
-        s.status = NB_Z_TIMEOUT;
-        done = true;
-      } else if (fresh) {
-        done = zone_init(t, s, w, P);
-        fresh = false;
-      } else {
-        done = zone_attempt(t, s, w, P);
-      }
-      if (done) {
-        zone_finish(t, s, w, P);
-        active = false;
-      }
+    if constexpr (in_step<NT>::value) {
+      // retired warps keep the block's phases
+      if (__syncthreads_and(retired)) break;
+    } else {
+      if (__all_sync(0xffffffffu, retired)) break;
+    }
+    const bool expired = active && P.budget_ns && gpu_ns() - t_start > P.budget_ns;
+    bool done = false;
+    if (expired && fresh) {
+      zone_timeout_unstarted(t, s.z, P);
+      active = false;
+    } else if (expired) {
+      s.status = NB_Z_TIMEOUT;
+      done = true;
+    }
+    const bool start = active && !expired && fresh;
+    const bool run = active && !expired && !fresh;
+    if (start) done = zone_init(t, s, w, P);
+    fresh = false;
+    if constexpr (in_step<NT>::value) {
+      done = zone_attempt(t, s, w, P, run) || done;
+    } else {
+      if (run) done = zone_attempt(t, s, w, P);
+    }
+    if (active && done) {
+      zone_finish(t, s, w, P);
+      active = false;
     }
   }
 }

@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <utility>
 #include <vector>
 
 #include "blob.h"
@@ -170,9 +171,21 @@ int build_blob(const nb_topology* T, const double* coeffs,
           if (F[k][j]) F[i][j] = 1;
   std::vector<std::vector<int>> slot(n, std::vector<int>(n, -1));
   int nnz = 0;
+  // the largest trailing block without a structural zero is stored dense
+  // (row by row) after the other slots
+  int tail = n;
+  while (tail > 0) {
+    bool full = true;
+    for (int j = tail - 1; j < n && full; ++j) full = F[tail - 1][j] && F[j][tail - 1];
+    if (!full) break;
+    --tail;
+  }
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j)
-      if (F[i][j]) slot[i][j] = nnz++;
+      if (F[i][j] && (i < tail || j < tail)) slot[i][j] = nnz++;
+  const int tail_slot = nnz;
+  for (int i = tail; i < n; ++i)
+    for (int j = tail; j < n; ++j) slot[i][j] = nnz++;
   // the pre-ordered LU may fill M's pattern to at most 4 times its nonzeros
   if (nnz > 32767 || nnz > 4 * nnz_jac) return NB_E_TOO_LARGE;
 
@@ -182,11 +195,13 @@ int build_blob(const nb_topology* T, const double* coeffs,
   std::vector<double> js_c;
   std::vector<uint8_t> js_flag(nnz, 0);
   {
-    int s = 0;
+    std::vector<std::pair<int, int>> at(nnz);
     for (int pi = 0; pi < n; ++pi)
-      for (int pj = 0; pj < n; ++pj) {
-        if (!F[pi][pj]) continue;
-        int i = perm[pi], j = perm[pj];
+      for (int pj = 0; pj < n; ++pj)
+        if (F[pi][pj]) at[slot[pi][pj]] = {pi, pj};
+    int s = 0;
+    for (const auto& e : at) {
+        int i = perm[e.first], j = perm[e.second];
         uint8_t fl = (i == j) ? SLOT_DIAG : 0;
         if (i < N && j < N) {
           for (int r = 0; r < R; ++r) {
@@ -430,6 +445,105 @@ int build_blob(const nb_topology* T, const double* coeffs,
     h.o_dej_ptr = B.add(dej_ptr);
     h.o_dej_d = B.add(dej_d);
   }
+  // ---- team programs (position space)
+  {
+    std::vector<uint32_t> cl, cu, cut, clt, ru, rlt;
+    std::vector<int32_t> cl_p(n + 1, 0), cu_p(n + 1, 0), cut_p(n + 1, 0), clt_p(n + 1, 0),
+        ru_p(n + 1, 0), rlt_p(n + 1, 0);
+    auto pk = [](int slot_, int row, int par) {
+      return (uint32_t)slot_ | ((uint32_t)(2 * row + par) << 16);
+    };
+    // rank of column k among row i's entries left of the diagonal, and of
+    // row k among column j's entries above it
+    auto lrank = [&](int i, int k) { int c = 0; for (int j = 0; j < k; ++j) c += F[i][j]; return c; };
+    auto urank = [&](int k, int j) { int c = 0; for (int i = 0; i < k; ++i) c += F[i][j]; return c; };
+    for (int k = 0; k < n; ++k) {
+      for (int i = k + 1; i < n; ++i) {
+        if (F[i][k]) cl.push_back(pk(slot[i][k], i, lrank(i, k) & 1));
+        if (F[k][i]) cut.push_back(pk(slot[k][i], i, urank(k, i) & 1));
+        if (F[k][i]) ru.push_back((uint32_t)slot[k][i] | ((uint32_t)i << 16));
+        if (F[i][k]) rlt.push_back((uint32_t)slot[i][k] | ((uint32_t)i << 16));
+      }
+      for (int i = 0; i < k; ++i) {
+        if (F[i][k]) cu.push_back(pk(slot[i][k], i, 0));
+        if (F[k][i]) clt.push_back(pk(slot[k][i], i, 0));
+      }
+      cl_p[k + 1] = (int32_t)cl.size();
+      cut_p[k + 1] = (int32_t)cut.size();
+      cu_p[k + 1] = (int32_t)cu.size();
+      clt_p[k + 1] = (int32_t)clt.size();
+      ru_p[k + 1] = (int32_t)ru.size();
+      rlt_p[k + 1] = (int32_t)rlt.size();
+    }
+    // rows of the back substitutions by dependency level (row k waits for
+    // the rows of its entries, all below it)
+    auto levels = [&](const std::vector<uint32_t>& es, const std::vector<int32_t>& ep,
+                      std::vector<int16_t>* rows, std::vector<int16_t>* lev) {
+      std::vector<int> lv(n, 0);
+      int top = 0;
+      for (int k = n - 1; k >= 0; --k) {
+        for (int e = ep[k]; e < ep[k + 1]; ++e)
+          lv[k] = std::max(lv[k], lv[es[e] >> 16] + 1);
+        top = std::max(top, lv[k]);
+      }
+      lev->push_back(0);
+      for (int l = 0; l <= top; ++l) {
+        for (int k = n - 1; k >= 0; --k)
+          if (lv[k] == l) rows->push_back((int16_t)k);
+        lev->push_back((int16_t)rows->size());
+      }
+    };
+    std::vector<int16_t> ru_row, ru_lev, rlt_row, rlt_lev;
+    levels(ru, ru_p, &ru_row, &ru_lev);
+    levels(rlt, rlt_p, &rlt_row, &rlt_lev);
+    h.n_ru_lev = (int32_t)ru_lev.size() - 1;
+    h.n_rlt_lev = (int32_t)rlt_lev.size() - 1;
+    h.o_cl = B.add(cl); h.o_cl_ptr = B.add(cl_p);
+    h.o_cu = B.add(cu); h.o_cu_ptr = B.add(cu_p);
+    h.o_cut = B.add(cut); h.o_cut_ptr = B.add(cut_p);
+    h.o_clt = B.add(clt); h.o_clt_ptr = B.add(clt_p);
+    h.o_ru = B.add(ru); h.o_ru_ptr = B.add(ru_p);
+    std::vector<int32_t> ru_tail(tail + 1);
+    for (int k = 0; k < tail; ++k) {
+      ru_tail[k] = ru_p[k + 1];
+      while (ru_tail[k] > ru_p[k] && (int)(ru[ru_tail[k] - 1] >> 16) >= tail) --ru_tail[k];
+    }
+    h.o_ru_tail = B.add(ru_tail);
+    h.o_ru_row = B.add(ru_row); h.o_ru_lev = B.add(ru_lev);
+    h.o_rlt = B.add(rlt); h.o_rlt_ptr = B.add(rlt_p);
+    h.o_rlt_row = B.add(rlt_row); h.o_rlt_lev = B.add(rlt_lev);
+    std::vector<int16_t> pos16(n), dpos(n);
+    for (int i = 0; i < n; ++i) pos16[i] = (int16_t)pos[i];
+    for (int k = 0; k < n; ++k) dpos[k] = (int16_t)slot[k][k];
+    h.o_pos = B.add(pos16);
+    h.o_dpos = B.add(dpos);
+    // gathers by decreasing length; those longer than 4 are split in two
+    auto by_length = [&](int cnt, const std::vector<int32_t>& ptr, const std::vector<uint8_t>* flag,
+                         std::vector<int16_t>* ord, int32_t* split, int32_t* fill) {
+      std::vector<int> idx(cnt);
+      for (int q = 0; q < cnt; ++q) idx[q] = q;
+      auto len = [&](int q) {
+        const int l = ptr[q + 1] - ptr[q];
+        return 2 * l + (flag && l == 0 && ((*flag)[q] & (SLOT_TROW | SLOT_TT)) ? 1 : 0);
+      };
+      std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return len(a) > len(b); });
+      *split = 0;
+      int nf = cnt;
+      for (int q = 0; q < cnt; ++q) {
+        ord->push_back((int16_t)idx[q]);
+        if (len(idx[q]) > 8) *split = q + 1;
+        if (len(idx[q]) == 0) nf = std::min(nf, q);
+      }
+      if (fill) *fill = nf;
+    };
+    std::vector<int16_t> js_ord, rhs_ord;
+    by_length(nnz, js_ptr, &js_flag, &js_ord, &h.js_split, &h.js_fill);
+    by_length(N, rhs_ptr, nullptr, &rhs_ord, &h.rhs_split, nullptr);
+    h.o_js_ord = B.add(js_ord);
+    h.o_rhs_ord = B.add(rhs_ord);
+    h.tail = tail;
+    h.tail_slot = tail_slot;
+  }
   h.nL = (int32_t)lslot.size(); h.nU = (int32_t)uslot.size(); h.nD = (int32_t)dslot.size();
   h.n_rhs = (int32_t)rhs_r.size(); h.n_js = (int32_t)js_src.size();
   h.n_fw = (int32_t)fw_s.size(); h.n_bw = (int32_t)bw_s.size();
@@ -459,6 +573,26 @@ int build_blob(const nb_topology* T, const double* coeffs,
   h.w_tmp = take(n); h.w_f0 = take(n);
   h.w_xh = take(HMAX * n); h.w_eh = take(HMAX); h.w_th = take(HMAX);
   h.lane_doubles = w;
+  // the same arrays as a team of threads keeps them: the solve vector and f
+  // (Newton loop) share room with the derivative terms (Jacobian)
+  w = 0;
+  h.th_x = take(n); h.th_xp = take(n); h.th_psi = take(n); h.th_iw = take(n);
+  h.th_tmp = take(n); h.th_pv = take(n);
+  h.th_k = take(R); h.th_rr = take(R);
+  h.th_g = h.th_kp = -1;
+  if (sh) { h.th_g = take(R); h.th_kp = take(R); }
+  h.th_lu = take(nnz);
+  h.th_eh = take(HMAX + 1); h.th_th = take(HMAX + 1);
+  const int dts = nd + (sh ? R : 0);
+  h.th_dt = take(std::max(dts, 4 * n));
+  h.th_y = h.th_dt;            // [2 n] partial sums, [n] solution
+  h.th_f = h.th_dt + 3 * n;
+  h.thot = w = (w + 1) & ~1;
+  w = 0;
+  h.tc_g = h.tc_kp = -1;
+  if (!sh) { h.tc_g = take(R); h.tc_kp = take(R); }
+  h.tc_f0 = take(n); h.tc_xh = take(HMAX * n);
+  h.tcold = w = (w + 1) & ~1;
 
   // algorithmic FP64 operation counts per event (an FMA counts 2 flops;
   // exp, log, cbrt, pow, sqrt and divisions are counted apart as special
