@@ -117,7 +117,7 @@ NB_HD inline void seg_start(const NT& t, AdjZone& Zs, WT& w, const AdjParams& A,
     // f(x0) for the first step's predictor, as the forward start-up forms it
     if (t.sh) eval_rates(t, s, w, t_powers(s.T9f, false, s.scr), s.T9f, false);
     eval_terms(t, w, w.xh);
-    eval_f(t, w, w.xh, w.f0);
+    eval_f(t, w, heat_rate(t, w, w.xh), w.f0);
   }
   Zs.lo = q0 + 1;
   Zs.rs = q0 + 1;
@@ -274,10 +274,11 @@ NB_HD inline bool adj_step(const NT& t, AdjZone& Zs, WT& w, const AT& a, const A
   vsync(t);
   if (t.sh) eval_rates(t, Zs.fz, w, t_powers(w.x[N], true, Zs.fz.scr), w.x[N], true);
   eval_terms(t, w, w.x);
-  assemble_M(t, w, w.x, alpha[0], h);
+  const HeatRate hr = heat_rate(t, w, w.x);
+  assemble_M(t, w, w.x, hr, alpha[0], h);
   factor_M(t, w);
   double icv = 0.0;
-  if (t.sh) icv = 1.0 / heat_capacity(t, w.x);
+  if (t.sh) icv = 1.0 / hr.cv;
   if (t.hasE) edot_gradient(t, w, a);
   const double ia0 = 1.0 / alpha[0];
   const int sl = ring(s);

@@ -249,6 +249,12 @@ int nb_net_get_info(nb_net net, nb_net_info* o) {
 
 // ------------------------------------------------------------------ specialised kernel
 
+// The variant a burn takes by itself: with x, d and f alone in registers it
+// spills nothing to speak of, and it ran fastest on every chain network and
+// size measured (self-heating, 65,536 zones: 331, 322, 312 ms for variants 1,
+// 2, 3).
+static constexpr int kBurnVariant = 3;
+
 // The specialised kernel of `variant` (1..3) for this network, generated,
 // compiled and loaded on first use.  Caller holds net->mu.
 static int spec_get(nb_net net, int variant, const void** fn) {
@@ -285,7 +291,7 @@ static void copy_log(const std::string& s, char* log, int64_t cap) {
 extern "C" int nb_net_specialize(nb_net net, int32_t variant, char* log, int64_t log_bytes) {
   if (!net || variant < 0 || variant > 3) return NB_E_ARG;
   std::lock_guard<std::mutex> lk(net->mu);
-  const int v = resolve_variant(net->h, variant);
+  const int v = variant > 0 ? variant : kBurnVariant;
   const void* fn = nullptr;
   const int rc = spec_get(net, v, &fn);
   copy_log(net->spec[v].log, log, log_bytes);
@@ -397,7 +403,7 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
       if (rc) return rc;
       spec_variant = o.specialize;
     } else if (specialize_auto_ok(net->h)) {
-      spec_variant = resolve_variant(net->h, 0);
+      spec_variant = kBurnVariant;
       if (spec_get(net, spec_variant, &spec_fn) != NB_OK) {
         spec_fn = nullptr;
         spec_variant = 0;
@@ -405,6 +411,20 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
     }
   }
   if (spec_fn) {
+    // A zone per lane while an SM's zones fit 256 lanes: a lane that gets a
+    // second zone ends long after the others (12,345 zones of the
+    // self-heating chain, 81 an SM: 64 threads 160 ms, 96 threads 108 ms).
+    // Past four warps, where every warp more slows the others, up to 5 % more
+    // zones than lanes are better: the last claimed are the shortest (20,000
+    // zones, 132 an SM: 128 threads 121 ms, 160 threads 140 ms).  Past 256 an
+    // SM the kernel packs its last zones
+    // (block_done), so the most lanes are the fastest: 65,536 zones take
+    // 344 ms with 128 threads, 311 ms with 256.
+    if (o.threads_per_block <= 0) {
+      const long long per_sm = (P.Z + net->sm_count - 1) / net->sm_count;
+      const long long lanes = per_sm <= 128 ? per_sm : per_sm * 20 / 21;
+      tpb = (int)std::min(256LL, (lanes + 31) / 32 * 32);
+    }
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, spec_fn, tpb, 0) != cudaSuccess) {
       cudaGetLastError();

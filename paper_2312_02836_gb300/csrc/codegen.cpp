@@ -68,17 +68,28 @@ struct Out {
   void raw(const std::string& t) { s += t; }
 };
 
-// pairs of a two-partial-sum gather over [beg, end): entries beg, beg+2, ..
-// go to a0 and beg+1, beg+3, .. to a1, except an odd last entry, which goes
-// to a0 (the order of the generic gather)
-template <class F>
-void emit_pairs(Out& o, int beg, int end, F term) {
-  int e = beg;
-  for (; e + 1 < end; e += 2) {
-    o("    a0 = %s;\n", term(e, "a0").c_str());
-    o("    a1 = %s;\n", term(e + 1, "a1").c_str());
+// c * src, without the product when c is +-1 (the same value)
+std::string product(double c, const std::string& src) {
+  if (c == 1.0) return src;
+  if (c == -1.0) return "-" + src;
+  return lit(c) + " * " + src;
+}
+
+// A two-partial-sum gather over [beg, end): entries beg, beg+2, .. go to a0
+// and beg+1, beg+3, .. to a1 (the order of the generic gather); the sum's
+// expression.  The generic sums start at 0; starting with the first product
+// drops two additions a sum (200 of the self-heating chain's 2,800 FP64
+// instructions an attempt) and can only change the sign of a zero.
+template <class C, class SRC>
+std::string emit_sum(Out& o, int beg, int end, C coef, SRC src) {
+  for (int e = beg; e < end; ++e) {
+    const char* a = (e - beg) & 1 ? "a1" : "a0";
+    if (e < beg + 2)
+      o("    double %s = %s;\n", a, product(coef(e), src(e)).c_str());
+    else
+      o("    %s = fma(%s, %s, %s);\n", a, lit(coef(e)).c_str(), src(e).c_str(), a);
   }
-  if (e < end) o("    a0 = %s;\n", term(e, "a0").c_str());
+  return end == beg ? "0.0" : end == beg + 1 ? "a0" : "a0 + a1";
 }
 
 }  // namespace
@@ -139,8 +150,10 @@ std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
       "typedef unsigned int uint32_t;\ntypedef unsigned long long uint64_t;\n"
       "#include \"expf64.cuh\"\n#include \"integrator.cuh\"\n\nnamespace nb {\n\n");
   o("struct GNet {\n  static constexpr int n = %d, N = %d, R = %d, sh = %d, hasE = %d;\n"
-    "  static constexpr double inv_n = 1.0 / %d;\n};\n\n",
-    n, N, R, sh ? 1 : 0, h.has_E ? 1 : 0, n);
+    "  static constexpr double inv_n = 1.0 / %d;\n"
+    "  static constexpr bool in_step = true;\n"
+    "  static constexpr int lane_doubles = %d;\n};\n\n",
+    n, N, R, sh ? 1 : 0, h.has_E ? 1 : 0, n, h.lane_doubles);
   const int Rd = R > 0 ? R : 1;
   const bool lu_reg = variant == 1, vec_reg = variant <= 2;
   const bool k_reg = sh;   // fixed-T rates live for the whole zone
@@ -151,7 +164,15 @@ std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
   else o("  LV lu;\n");
   if (k_reg) o("  double k[%d], g[%d], kp[%d];\n", Rd, Rd, Rd);
   else o("  LV k;\n");
-  o("  LV f0, xh, eh, th;\n};\n\n");
+  // take: a zone's arrays that outlive an attempt, from the lane d doubles on
+  o("  LV f0, xh, eh, th;\n  __device__ void take(long long d) {\n"
+    "    for (int e = 0; e < %d; ++e) f0.p[e * WS_LANES] = f0.p[e * WS_LANES + d];\n"
+    "    for (int e = 0; e < %d; ++e) xh.p[e * WS_LANES] = xh.p[e * WS_LANES + d];\n"
+    "    for (int e = 0; e < HMAX; ++e) {\n      eh.p[e * WS_LANES] = eh.p[e * WS_LANES + d];\n"
+    "      th.p[e * WS_LANES] = th.p[e * WS_LANES + d];\n    }\n", n, HMAX * n);
+  if (!k_reg)
+    o("    for (int e = 0; e < %d; ++e) k.p[e * WS_LANES] = k.p[e * WS_LANES + d];\n", R);
+  o("  }\n};\n\n");
 
   // ---- rate tables (grid, ln lambda at the nodes, charges) as literal arrays
   const bool has_tab = h.n_tab > 0;
@@ -300,30 +321,31 @@ std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
   o("}\n\n");
 
   // ---- edot
-  o("NB_HD __forceinline__ double eval_edot(const GNet&, GWS& w) {\n"
-    "  double a0 = 0.0, a1 = 0.0;\n");
-  emit_pairs(o, 0, R, [&](int r, const char* acc) {
-    return "fma(" + lit(Q[r]) + ", w.rr[" + std::to_string(r) + "], " + acc + ")";
-  });
-  o("  return a0 + a1;\n}\n\n");
+  auto rr = [&](int r) { return "w.rr[" + std::to_string(r) + "]"; };
+  o("NB_HD __forceinline__ double eval_edot(const GNet&, GWS& w) {\n");
+  {
+    const std::string sum = emit_sum(o, 0, R, [&](int r) { return Q[r]; }, rr);
+    o("  return %s;\n}\n\n", sum.c_str());
+  }
 
   // ---- f
-  o("template <class V, class O>\nNB_HD __forceinline__ void eval_f(const GNet& t, GWS& w,"
-    " const V& v, O&& out) {\n");
+  o("template <class O>\nNB_HD __forceinline__ void eval_f(const GNet& t, GWS& w,"
+    " const HeatRate& hr, O&& out) {\n");
   for (int i = 0; i < N; ++i) {
-    o("  {\n    double a0 = 0.0, a1 = 0.0;\n");
-    emit_pairs(o, rhs_ptr[i], rhs_ptr[i + 1], [&](int e, const char* acc) {
-      return "fma(" + lit(rhs_c[e]) + ", w.rr[" + std::to_string(rhs_r[e]) + "], " + acc + ")";
-    });
-    o("    out[%d] = a0 + a1;\n  }\n", i);
+    o("  {\n");
+    const std::string sum = emit_sum(o, rhs_ptr[i], rhs_ptr[i + 1],
+                                     [&](int e) { return rhs_c[e]; },
+                                     [&](int e) { return rr(rhs_r[e]); });
+    o("    out[%d] = %s;\n  }\n", i, sum.c_str());
   }
-  if (sh) o("  out[%d] = eval_edot(t, w) / heat_capacity(t, v);\n", N);
+  if (sh) o("  out[%d] = hr.ed / hr.cv;\n", N);
   o("}\n\n");
 
   // ---- M = alpha0 I - h J
   const int ndt = nd + (sh ? R : 0);
   o("template <class V>\nNB_HD __forceinline__ void assemble_M(const GNet& t, GWS& w,"
-    " const V& v, double alpha0, double h) {\n  double dt[%d];\n", ndt > 0 ? ndt : 1);
+    " const V& v, const HeatRate& hr, double alpha0, double h) {\n  double dt[%d];\n",
+    ndt > 0 ? ndt : 1);
   for (int d = 0; d < nd; ++d) {
     o("  dt[%d] = w.k[%d] * %s", d, dt_r[d], lit(dt_m[d]).c_str());
     if (dt_o[2 * d] >= 0) o(" * v[%d]", dt_o[2 * d]);
@@ -332,16 +354,21 @@ std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
   }
   if (sh) {
     for (int r = 0; r < R; ++r) o("  dt[%d] = w.rr[%d] * w.g[%d];\n", nd + r, r, r);
-    o("  const TRow tr = t_row(eval_edot(t, w), heat_capacity(t, v), v[%d]);\n", N);
+    o("  const TRow tr = t_row(hr.ed, hr.cv, v[%d]);\n", N);
   }
   o("  const double mh = -h;\n");
   for (int s = 0; s < nnz; ++s) {
-    o("  {\n    double a0 = 0.0, a1 = 0.0;\n");
-    emit_pairs(o, js_ptr[s], js_ptr[s + 1], [&](int e, const char* acc) {
-      return "fma(" + lit(js_c[e]) + ", dt[" + std::to_string(js_src[e]) + "], " + acc + ")";
-    });
-    o("    double acc = a0 + a1;\n");
     const uint8_t fl = js_flag[s];
+    if (js_ptr[s] == js_ptr[s + 1] && !(fl & (SLOT_TROW | SLOT_TT))) {
+      // fill: -h times an empty sum
+      o("  w.lu[%d] = %s;\n", s, fl & SLOT_DIAG ? "alpha0" : "-0.0");
+      continue;
+    }
+    o("  {\n");
+    const std::string sum = emit_sum(o, js_ptr[s], js_ptr[s + 1],
+                                     [&](int e) { return js_c[e]; },
+                                     [&](int e) { return "dt[" + std::to_string(js_src[e]) + "]"; });
+    o("    double acc = %s;\n", sum.c_str());
     if (fl & SLOT_TROW) o("    acc = fma(acc, tr.a1, tr.b1);\n");
     else if (fl & SLOT_TT) o("    acc = fma(acc, tr.a1, tr.b2);\n");
     o("    double m = mh * acc;\n");
@@ -379,12 +406,15 @@ std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
   auto tri = [&](const TriRow* rows, const int16_t* es, const int16_t* ec) {
     for (int q = 0; q < n; ++q) {
       const TriRow& r = rows[q];
-      o("  {\n    double a0 = v[%d], a1 = 0.0;\n", r.tgt);
-      emit_pairs(o, r.beg, r.end, [&](int e, const char* acc) {
-        return "fma(-w.lu[" + std::to_string(es[e]) + "], v[" + std::to_string(ec[e]) + "], " +
-               acc + ")";
-      });
-      o("    double acc = a0 + a1;\n");
+      o("  {\n    double a0 = v[%d];\n", r.tgt);
+      for (int e = r.beg; e < r.end; ++e) {
+        const int q = e - r.beg;
+        if (q == 1)
+          o("    double a1 = -(w.lu[%d] * v[%d]);\n", es[e], ec[e]);
+        else
+          o("    a%d = fma(-w.lu[%d], v[%d], a%d);\n", q & 1, es[e], ec[e], q & 1);
+      }
+      o("    double acc = a0%s;\n", r.end - r.beg > 1 ? " + a1" : "");
       if (r.dslot >= 0) o("    acc *= w.lu[%d];\n", r.dslot);
       o("    v[%d] = acc;\n  }\n", r.tgt);
     }

@@ -354,8 +354,8 @@ __device__ __forceinline__ void gather_rows(const TNet<P, S, D>& t, const int16_
 }
 
 template <int P, int S, class D>
-__device__ __forceinline__ void eval_f(const TNet<P, S, D>& t, const CWS& w, const CV& v,
-                                       const CV& out) {
+__device__ __forceinline__ void eval_f(const TNet<P, S, D>& t, const CWS& w,
+                                       const HeatRate& hr, const CV& out) {
   t.sync();
   const BlobHeader& h = t.h;
   gather_rows(t, t.template arr<int16_t>(h.o_rhs_ord), h.rhs_split, t.N,
@@ -363,7 +363,7 @@ __device__ __forceinline__ void eval_f(const TNet<P, S, D>& t, const CWS& w, con
               t.template arr<double>(h.o_rhs_c), w.rr,
               [&](int i, double a) { out[i] = a; });
   if (t.sh) {
-    const double fT = eval_edot(t, w) / heat_capacity(t, v);
+    const double fT = hr.ed / hr.cv;
     if (t.lane == 0) out[t.N] = fT;
   }
   t.sync();
@@ -372,7 +372,7 @@ __device__ __forceinline__ void eval_f(const TNet<P, S, D>& t, const CWS& w, con
 // M = alpha0 I - h J(v) into w.lu (needs w.k, w.g (self-heating), w.rr at v)
 template <int P, int S, class D>
 __device__ __forceinline__ void assemble_M(const TNet<P, S, D>& t, const CWS& w, const CV& v,
-                                           double alpha0, double h) {
+                                           const HeatRate& hr, double alpha0, double h) {
   t.sync();
   const BlobHeader& hd = t.h;
   const int nd = hd.nd;
@@ -391,7 +391,7 @@ __device__ __forceinline__ void assemble_M(const TNet<P, S, D>& t, const CWS& w,
   TRow tr{0.0, 0.0, 0.0};
   if (t.sh) {
     for (int r = t.lane; r < t.R; r += P) w.dt[nd + r] = w.rr[r] * w.g[r];
-    tr = t_row(eval_edot(t, w), heat_capacity(t, v), v[t.N]);
+    tr = t_row(hr.ed, hr.cv, v[t.N]);
   }
   t.sync();
   const double mh = -h;

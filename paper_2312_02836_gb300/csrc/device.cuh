@@ -296,16 +296,16 @@ NB_HD __forceinline__ double gather2(const double* c, const TI* idx, int beg, in
   return a0 + a1;
 }
 
-// out = f(v) given w.rr for v
-NB_HD inline void eval_f(const Net& t, const WS& w, const LV& v, const LV& out) {
+// out = f given w.rr and the heat rate
+NB_HD inline void eval_f(const Net& t, const WS& w, const HeatRate& hr, const LV& out) {
 #pragma unroll 2
   for (int i = 0; i < t.N; ++i)
     out[i] = gather2(t.rhs_c, t.rhs_r, t.rhs_ptr[i], t.rhs_ptr[i + 1], w.rr);
-  if (t.sh) out[t.N] = eval_edot(t, w) / heat_capacity(t, v);
+  if (t.sh) out[t.N] = hr.ed / hr.cv;
 }
 
 // M = alpha0 I - h J(v) into w.lu (needs w.k, w.g (self-heating), w.rr at v)
-NB_HD inline void assemble_M(const Net& t, const WS& w, const LV& v,
+NB_HD inline void assemble_M(const Net& t, const WS& w, const LV& v, const HeatRate& hr,
                              double alpha0, double h) {
 #pragma unroll 4
   for (int d = 0; d < t.nd; ++d) {
@@ -318,7 +318,7 @@ NB_HD inline void assemble_M(const Net& t, const WS& w, const LV& v,
   TRow tr{0.0, 0.0, 0.0};
   if (t.sh) {
     for (int r = 0; r < t.R; ++r) w.dt[t.nd + r] = w.rr[r] * w.g[r];
-    tr = t_row(eval_edot(t, w), heat_capacity(t, v), v[t.N]);
+    tr = t_row(hr.ed, hr.cv, v[t.N]);
   }
   const double mh = -h;
 #pragma unroll 2

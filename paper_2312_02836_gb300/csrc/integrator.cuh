@@ -16,9 +16,9 @@
 //                                     tables, from its initial composition
 //   eval_rates_near(t, s, w, T9, ref, T9ref)  k_r from kp_r (rate_near)
 //   eval_terms(t, w, v)               rr_r = k_r prod Y of the reactants
-//   eval_f(t, w, v, out)              out = f(v) from rr
+//   eval_f(t, w, hr, out)             out = f from rr and the heat rate hr
 //   eval_edot(t, w)                   sum_r Q_r rr_r
-//   assemble_M(t, w, v, alpha0, h)    lu = alpha0 I - h J(v)
+//   assemble_M(t, w, v, hr, alpha0, h)  lu = alpha0 I - h J(v)
 //   factor_M(t, w)                    static-pivot LU of lu in place
 //   solve_M(t, w, v)                  v <- M^-1 v with the factored lu
 // Three network types exist: the generic one (device.cuh) walks a compiled
@@ -98,10 +98,8 @@ NB_HD __forceinline__ bool vlead(const NT& t) {
   if constexpr (is_coop<NT>::value) return t.lane == 0; else return true;
 }
 
-// Network types whose warps of a block run the step's phases together (the
-// generated kernel: its straight-line code is larger than the instruction
-// caches, and a block's warps share what they fetch only while they are in
-// the same part of it)
+// Network types whose warps of a block start their attempts together
+// (block_done; the generated kernel)
 template <class NT, class = void>
 struct in_step {
   static constexpr bool value = false;
@@ -110,20 +108,6 @@ template <class NT>
 struct in_step<NT, decltype((void)NT::in_step)> {
   static constexpr bool value = NT::in_step;
 };
-template <class NT>
-NB_HD __forceinline__ void phase_sync(const NT&) {
-#ifdef __CUDA_ARCH__
-  if constexpr (in_step<NT>::value) __syncthreads();
-#endif
-}
-// does this thread (with phases in step: any thread of the block) go on?
-template <class NT>
-NB_HD __forceinline__ bool phase_any(const NT&, bool go) {
-#ifdef __CUDA_ARCH__
-  if constexpr (in_step<NT>::value) return __syncthreads_or(go) != 0;
-#endif
-  return go;
-}
 
 // lane-strided view of one per-lane array
 struct LV {
@@ -505,6 +489,21 @@ NB_HD __forceinline__ TRow t_row(double ed, double cv, double T9) {
   return r;
 }
 
+// edot and c_v at a state (self-heating): the T9 equation is edot / c_v
+struct HeatRate {
+  double ed, cv;
+};
+
+template <class NT, class WT, class V>
+NB_HD __forceinline__ HeatRate heat_rate(const NT& t, WT& w, const V& v) {
+  HeatRate q{0.0, 0.0};
+  if (t.sh) {
+    q.ed = eval_edot(t, w);
+    q.cv = heat_capacity(t, v);
+  }
+  return q;
+}
+
 // ---------------------------------------------------------------- integrator
 
 // ||v||^2 = mean (v_i * iw_i)^2, two interleaved partial sums (the tests
@@ -799,7 +798,7 @@ NB_HD __forceinline__ bool zone_init(const NT& t, Zone& s, WT& w, const BurnPara
   eval_rates(t, s, w, t_powers(s.T9f, false, s.scr), s.T9f, false);
   s.c_teval++;
   eval_terms(t, w, x0);
-  eval_f(t, w, x0, w.f0);
+  eval_f(t, w, heat_rate(t, w, x0), w.f0);
   s.c_rhs++;
   NB_UNROLL
   for (int r = vbeg(t); r < t.R; r += vstep(t)) fin = fin && finite_bits(w.k[r]);
@@ -832,7 +831,7 @@ NB_HD __forceinline__ bool zone_init(const NT& t, Zone& s, WT& w, const BurnPara
     s.c_teval++;
   }
   eval_terms(t, w, w.x);
-  eval_f(t, w, w.x, w.f);
+  eval_f(t, w, heat_rate(t, w, w.x), w.f);
   s.c_rhs++;
   const double ihp = 1.0 / hp;
   vsync(t);
@@ -865,8 +864,9 @@ struct Attempt {
 // and, when it accepts, the energy rate.  Leaves the solution in w.x, the
 // predictor in w.xp and alpha_0..alpha_kk in alpha.  The forward burn and the
 // adjoint's recomputation of checkpointed segments both run it, so that they
-// produce the same bits.  Threads without an attempt pass run = false and
-// only keep the phases of their block.
+// produce the same bits.  With run unset nothing is done: the phases test it
+// one by one, which keeps a warp's lanes together (4,096 zones of the
+// 13-species chain take 57.8 ms with the call itself under the test, 52.7 so).
 template <bool FULL, class NT, class WT>
 NB_HD __forceinline__ Attempt attempt_solve(const NT& t, Zone& s, WT& w, bool run, double atol,
                                             double rtol, double h, double t_new, int kk,
@@ -888,7 +888,6 @@ NB_HD __forceinline__ Attempt attempt_solve(const NT& t, Zone& s, WT& w, bool ru
     for (int i = vbeg(t); i < n; i += vstep(t)) w.x[i] = w.xp[i];
     vsync(t);
   }
-  phase_sync(t);
   // Jacobian at the predictor, M, LU; with self-heating the predictor's
   // temperature is the attempt's reference for the rates
   double Tref = 0.0;
@@ -903,9 +902,11 @@ NB_HD __forceinline__ Attempt attempt_solve(const NT& t, Zone& s, WT& w, bool ru
     }
     eval_terms(t, w, w.x);
   }
-  phase_sync(t);
+  // the first Newton pass is at the predictor too: it takes these
+  HeatRate hr{0.0, 0.0};
   if (run) {
-    assemble_M(t, w, w.x, alpha[0], h);
+    hr = heat_rate(t, w, w.x);
+    assemble_M(t, w, w.x, hr, alpha[0], h);
     s.c_jac++;
     at.lu_ok = factor_M(t, w);
   }
@@ -913,19 +914,20 @@ NB_HD __forceinline__ Attempt attempt_solve(const NT& t, Zone& s, WT& w, bool ru
   // of the solution for the energy, from the one place in the code that does
   bool go = run && at.lu_ok, energy = false;
   double nrm_prev = 0.0;
-  for (int m = 0; phase_any(t, go); ++m) {
-    if (!go) continue;
+  for (int m = 0; go; ++m) {
     if (m > 0) {
       if (t.sh) { eval_rates_near(t, s, w, w.x[N], pref, Tref); s.c_teval++; }
       eval_terms(t, w, w.x);
+      if (t.sh) hr.ed = eval_edot(t, w);
     }
     if (energy) {
-      at.ed = eval_edot(t, w);
+      at.ed = t.sh ? hr.ed : eval_edot(t, w);
       s.c_edot++;
       go = false;
       continue;
     }
-    eval_f(t, w, w.x, w.f);
+    if (t.sh && m > 0) hr.cv = heat_capacity(t, w.x);
+    eval_f(t, w, hr, w.f);
     s.c_rhs++;
     const double nrm2 = newton_correct(t, w, alpha[0], h);
     s.c_newton++;
@@ -957,32 +959,23 @@ NB_HD __forceinline__ Attempt attempt_solve(const NT& t, Zone& s, WT& w, bool ru
   return at;
 }
 
-// The factor on h after an accepted step: when the zone may change its order
-// (sel), the best of orders k-1, k, k+1, else that of the step's own order kk.
+// One step attempt.  Returns true when the zone is finished.  Written with one
+// exit: the lanes of a warp meet again after every decision, where early
+// returns keep those that take them apart (4,096 zones of the 13-species
+// chain: 57.5 ms with returns).
 template <class NT, class WT>
-NB_HD __forceinline__ double next_factor(const NT& t, const Zone& s, WT& w, bool acc, bool sel,
-                                         double err2, double h, int kk, int& best_q) {
-  best_q = s.k;
-  if (!acc) return 1.0;
-  return sel ? order_factor(t, s, w, err2, h, best_q) : step_factor(err2, kk);
-}
-
-// One step attempt of a thread with run set.  Returns true when its zone is
-// finished.
-template <class NT, class WT>
-NB_HD __forceinline__ bool zone_attempt(const NT& t, Zone& s, WT& w, const BurnParams& P,
-                                        bool run = true) {
+NB_HD __forceinline__ bool zone_attempt(const NT& t, Zone& s, WT& w, const BurnParams& P) {
   const int n = t.n;
   bool done = false;
   double h = s.h;
-  if (run && s.c_acc + s.c_rej_err + s.c_rej_newton >= P.max_attempts) {
+  if (s.c_acc + s.c_rej_err + s.c_rej_newton >= P.max_attempts) {
     s.status = NB_Z_MAX_STEPS;
     done = true;
-  } else if (run && (h < 1e-30 * s.tend || h < 1e-14 * s.t)) {
+  } else if (h < 1e-30 * s.tend || h < 1e-14 * s.t) {
     s.status = NB_Z_DT_UNDERFLOW;
     done = true;
   }
-  run = run && !done;
+  const bool run = !done;
   double t_new;
   if (s.t + h >= s.tend) { h = s.tend - s.t; t_new = s.tend; }
   else t_new = s.t + h;
@@ -1044,8 +1037,11 @@ NB_HD __forceinline__ bool zone_attempt(const NT& t, Zone& s, WT& w, const BurnP
   }
   // next step size and order
   if (acc) s.nconsec++;
-  int best_q;
-  double factor = next_factor(t, s, w, acc, acc && s.nconsec >= s.k + 1, at.err2, h, kk, best_q);
+  int best_q = s.k;
+  double factor = 1.0;
+  if (acc)
+    factor = s.nconsec >= s.k + 1 ? order_factor(t, s, w, at.err2, h, best_q)
+                                  : step_factor(at.err2, kk);
   if (acc) {
     if (best_q != s.k) { s.k = best_q; s.nconsec = 0; }
     if (factor < 0.2) factor = 0.2;
@@ -1129,6 +1125,69 @@ NB_HD __forceinline__ void zone_finish(const NT& t, const Zone& s, const WT& w,
   }
 }
 
+#ifdef __CUDA_ARCH__
+// The barrier at which a block's warps start their attempts together, and,
+// once the queue is empty, the packing of its last zones.  True when the
+// block has none left.
+//  * The generated kernel is straight-line code larger than the instruction
+//    caches; warps that run the same part of it at one time share what they
+//    fetch (65,536 zones of the self-heating chain: 412 -> 360 ms with the
+//    barrier alone; barriers inside the attempt gained no more).
+//  * A warp's FP64 instruction costs the same for 1 and for 32 lanes, and a
+//    block's last zones are spread over all its warps.  So when the zones of
+//    one warp fit into the idle lanes of the others, they move there (their
+//    history is in the workspace, the rest is the Zone struct) and the warp
+//    stops.  Taken first: a warp of the scheduler with the most running
+//    warps, then the one with the fewest zones.
+template <class NT, class WT>
+__device__ __forceinline__ bool block_done(const NT&, WT& w, Zone& s, bool& active,
+                                           bool& retired, bool& fresh) {
+  __shared__ int cnt[8];        // running zones of each warp
+  __shared__ Zone moved[32];
+  __shared__ int from[32];      // thread | fresh << 16
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const unsigned on = __ballot_sync(0xffffffffu, active), below = (1u << lane) - 1u;
+  if (lane == 0) cnt[warp] = __popc(on);
+  if (!__syncthreads_or(retired)) return false;
+  int total = 0, running = 0, load[4] = {0, 0, 0, 0};
+  for (int v = 0; v < nw; ++v) {
+    total += cnt[v];
+    running += cnt[v] > 0;
+    load[v & 3] += cnt[v] > 0;
+  }
+  if (total == 0) return true;
+  int take = -1, best = 1 << 30;
+  for (int v = 0; v < nw; ++v) {
+    const int key = cnt[v] - 64 * load[v & 3];
+    if (cnt[v] > 0 && total <= 32 * (running - 1) && key < best) { best = key; take = v; }
+  }
+  if (take >= 0) {
+    if (warp == take && active) {
+      const int q = __popc(on & below);
+      moved[q] = s;
+      from[q] = threadIdx.x | (fresh ? 1 << 16 : 0);
+      active = false;
+      retired = true;
+    }
+    __syncthreads();
+    if (warp != take && cnt[warp] > 0 && !active) {
+      int q = __popc(~on & below);   // rank among the idle lanes
+      for (int v = 0; v < warp; ++v)
+        if (v != take && cnt[v] > 0) q += 32 - cnt[v];
+      if (q < cnt[take]) {
+        s = moved[q];
+        fresh = from[q] >> 16;
+        active = true;
+        const int src = from[q] & 0xffff;
+        w.take((long long)((src >> 5) - warp) * NT::lane_doubles * WS_LANES + (src & 31) - lane);
+      }
+    }
+    __syncthreads();   // cnt, moved and the arrays of the old lanes are free
+  }
+  return false;
+}
+#endif
+
 // The persistent lane-per-zone loop: every lane claims zones from the device
 // queue (one atomic per warp for all lanes that need a zone), initialises,
 // attempts steps and writes each zone back, and claims the next one as soon
@@ -1162,8 +1221,7 @@ __device__ __forceinline__ void burn_claim_loop(const NT& t, WT& w, const BurnPa
       }
     }
     if constexpr (in_step<NT>::value) {
-      // retired warps keep the block's phases
-      if (__syncthreads_and(retired)) break;
+      if (block_done(t, w, s, active, retired, fresh)) break;
     } else {
       if (__all_sync(0xffffffffu, retired)) break;
     }
@@ -1176,15 +1234,10 @@ __device__ __forceinline__ void burn_claim_loop(const NT& t, WT& w, const BurnPa
       s.status = NB_Z_TIMEOUT;
       done = true;
     }
-    const bool start = active && !expired && fresh;
-    const bool run = active && !expired && !fresh;
+    const bool start = active && !expired && fresh, run = active && !expired && !fresh;
     if (start) done = zone_init(t, s, w, P);
     fresh = false;
-    if constexpr (in_step<NT>::value) {
-      done = zone_attempt(t, s, w, P, run) || done;
-    } else {
-      if (run) done = zone_attempt(t, s, w, P);
-    }
+    if (run) done = zone_attempt(t, s, w, P);
     if (active && done) {
       zone_finish(t, s, w, P);
       active = false;
