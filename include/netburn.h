@@ -154,20 +154,22 @@ typedef struct {
   int32_t specialize_auto;  /* 1: burns with options.specialize = 0 use the
                                network-specialised kernel (when it builds) */
   int32_t last_specialized; /* storage variant of the specialised kernel the
-                               last burn ran, 0 = a generic kernel */
+                               last burn ran (its team form counts as the
+                               variant it stands in for), 0 = a generic
+                               kernel */
   int32_t reserved;
 } nb_net_info;
 
 typedef struct {
   int32_t max_attempts;     /* step attempts per zone (default 500000) */
   int32_t kernel;           /* NB_KERNEL_* */
-  int32_t threads_per_block;/* 0 = 128; a multiple of 32, at most 256
-                               (128 for the plain kernel) */
-  int32_t blocks_per_sm;    /* 0 = library choice (persistent kernel); the
-                               warp kernel (NB_KERNEL_COOP) with >= 3 and
-                               threads_per_block <= 128 runs its variant
-                               built for three blocks per SM (registers
-                               capped at 168) */
+  int32_t threads_per_block;/* 0 = library choice, from the number of zones;
+                               a multiple of 32, at most 256 (128 for the
+                               plain kernel) */
+  int32_t blocks_per_sm;    /* 0 = library choice; at most that many blocks
+                               per SM.  With NB_KERNEL_COOP the two bound the
+                               zones in flight; how many threads share a zone
+                               follows the network and the number of zones */
   int32_t blob_in_shared;   /* -1 auto, 0 global (L1), 1 shared memory */
   int32_t ws_in_shared;     /* persistent kernel: the first ws_in_shared warps
                                of each block keep their Newton-loop arrays in
@@ -185,7 +187,9 @@ typedef struct {
                                0 (default) automatic: the kernel generated
                                for this network (see nb_net_specialize) when
                                the network is small enough for it and it
-                               builds, else the generic kernel; -1 always the
+                               builds (a few lanes per zone while there are
+                               few zones and no launch shape is asked for,
+                               else one), else the generic kernel; -1 always the
                                generic kernel; 1..3 the specialised kernel
                                with that storage variant (NB_E_COMPILE when it
                                cannot be built).  Ignored with ws_in_shared

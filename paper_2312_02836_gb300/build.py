@@ -17,6 +17,7 @@ HEADERS = ["blob.h", "device.cuh", "integrator.cuh", "adjoint.cuh", "coop.cuh", 
 # headers the run-time compiler needs, embedded as text into the library
 # (name as written in the #include directive, path)
 EMBED = [("expf64.cuh", "csrc/expf64.cuh"), ("integrator.cuh", "csrc/integrator.cuh"),
+         ("device.cuh", "csrc/device.cuh"), ("coop.cuh", "csrc/coop.cuh"),
          ("blob.h", "csrc/blob.h"), ("../../include/netburn.h", "../include/netburn.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -255,18 +255,22 @@ int nb_net_get_info(nb_net net, nb_net_info* o) {
 // 2, 3).
 static constexpr int kBurnVariant = 3;
 
-// The specialised kernel of `variant` (1..3) for this network, generated,
-// compiled and loaded on first use.  Caller holds net->mu.
+// The specialised kernel of `variant` (an index of net->spec) for this
+// network, generated, compiled and loaded on first use.  Caller holds net->mu.
 static int spec_get(nb_net net, int variant, const void** fn) {
   nb_net_s::Spec& sp = net->spec[variant];
   if (sp.state == 0) {
     std::vector<char> cubin;
-    const std::string src = specialized_source(net->blob, variant);
+    const bool team = variant >= nb_net_s::kSpecTeam;
+    const std::string src =
+        team ? specialized_team_source(net->blob, 8 << (variant - nb_net_s::kSpecTeam))
+             : specialized_source(net->blob, variant);
+    const char* name = team ? "nb_spec_team" : "nb_spec_burn";
     int rc = compile_specialized(src, &cubin, &sp.log, false);
     if (rc == NB_OK &&
         (cudaLibraryLoadData(&sp.lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) !=
              cudaSuccess ||
-         cudaLibraryGetKernel(&sp.kern, sp.lib, "nb_spec_burn") != cudaSuccess)) {
+         cudaLibraryGetKernel(&sp.kern, sp.lib, name) != cudaSuccess)) {
       cudaGetLastError();
       if (sp.lib) cudaLibraryUnload(sp.lib);
       sp.lib = nullptr;
@@ -363,6 +367,64 @@ int nb::schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaS
   return NB_OK;
 }
 
+// Lanes per zone of the generated kernel's team form, 0 for a zone per lane.
+// With few zones per SM the longest zone sets the time, and its FP64
+// instructions are what a team spreads: 64 zones of the self-heating chain
+// take 94 ms with one lane each, 47, 39, 36 ms with 8, 16, 32. A team costs
+// an SM more instructions per zone, though, so the more zones the fewer
+// lanes: 500 zones 99 / 49 / 41 / 38 ms; 1,500 (10 an SM) 100 / 50 / 44 /
+// 67; 4,096 (27) 100 / 59 / 92 / 144; 8,192 (54) 101 / 116 / 160 / 267. The
+// fixed-temperature, tabulated and effective-rate chains cross between 38
+// and 60 an SM. A launch shape asked for is a lane kernel's.
+static int spec_team_lanes(nb_net net, const BurnParams& P, const nb_options& o) {
+  if (o.threads_per_block > 0 || o.blocks_per_sm > 0) return 0;
+  const long long sm = net->sm_count;
+  return P.Z <= 5 * sm ? 32 : P.Z <= 12 * sm ? 16 : P.Z <= 40 * sm ? 8 : 0;
+}
+
+// Burn few zones of a network with a generated kernel on its team form (8, 16
+// or 32 lanes a zone); false when it can't be built or doesn't fit.
+static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int lanes,
+                             cudaStream_t st, int* rc) {
+  const int idx = nb_net_s::kSpecTeam + (lanes == 8 ? 0 : lanes == 16 ? 1 : 2);
+  // doubles between teams: 8 mod 16, so that two teams' like accesses fall in
+  // different halves of the shared-memory banks
+  const int stride = (net->h.thot + net->h.tcold + 7) / 16 * 16 + 8;
+  const size_t blob_b = (size_t)net->h.bytes, team_b = (size_t)stride * sizeof(double);
+  const long long per_sm = (P.Z + net->sm_count - 1) / net->sm_count;
+  int threads = (int)std::min<long long>(256, (per_sm * lanes + 31) / 32 * 32);
+  while (threads > 32 && blob_b + threads / lanes * team_b > net->smem_optin) threads -= 32;
+  const size_t dyn = blob_b + threads / lanes * team_b;
+  const void* fn = nullptr;
+  if (dyn > net->smem_optin || spec_get(net, idx, &fn) != NB_OK) return false;
+  int occ = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, dyn) != cudaSuccess || occ < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  const int teams = threads / lanes;
+  const long long blocks =
+      std::min<long long>((long long)occ * net->sm_count, (P.Z + teams - 1) / teams);
+  const long long elanes = nb::prepass_lanes(net, P.Z);
+  *rc = nb::ensure((void**)&net->ws, &net->ws_bytes,
+                   (size_t)elanes * net->h.lane_doubles * sizeof(double));
+  if (*rc) return true;
+  P.ws = net->ws;
+  P.queue = net->queue;
+  P.smem_warps = stride;
+  P.order = nullptr;
+  if (o.schedule == 1 && P.Z > blocks * teams) {   // else every zone starts at once
+    *rc = nb::schedule_longest_first(net, P, elanes, st);
+    if (*rc) return true;
+  }
+  void* args[] = {&P};
+  *rc = cudaMemsetAsync(net->queue, 0, sizeof(unsigned long long), st) == cudaSuccess &&
+                cudaLaunchKernel(fn, dim3((unsigned)blocks), dim3(threads), args, dyn, st) == cudaSuccess
+            ? NB_OK : NB_E_CUDA;
+  return true;
+}
+
 // Launch one burn (device pointers).  Caller holds net->mu.
 static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
                        cudaStream_t st) {
@@ -403,6 +465,12 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
       if (rc) return rc;
       spec_variant = o.specialize;
     } else if (specialize_auto_ok(net->h)) {
+      int rc = NB_OK;
+      if (const int lanes = spec_team_lanes(net, P, o); lanes > 0 &&
+          launch_spec_team(net, P, o, lanes, st, &rc)) {
+        net->last_spec = kBurnVariant;
+        return rc;
+      }
       spec_variant = kBurnVariant;
       if (spec_get(net, spec_variant, &spec_fn) != NB_OK) {
         spec_fn = nullptr;

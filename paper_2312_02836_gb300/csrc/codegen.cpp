@@ -440,6 +440,41 @@ std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
   return o.s;
 }
 
+std::string specialized_team_source(const std::vector<uint8_t>& blob, int threads) {
+  const BlobHeader& h = *reinterpret_cast<const BlobHeader*>(blob.data());
+  Out o;
+  o("// network-specialised team kernel: n = %d, R = %d, LU slots %d, %d threads per zone\n", h.n,
+    h.R, h.nnz, threads);
+  o.raw(
+      "typedef signed char int8_t;\ntypedef short int16_t;\ntypedef int int32_t;\n"
+      "typedef long long int64_t;\ntypedef unsigned char uint8_t;\n"
+      "typedef unsigned int uint32_t;\ntypedef unsigned long long uint64_t;\n"
+      "typedef unsigned long size_t;\n"
+      "#include \"coop.cuh\"\n\nnamespace nb {\n\n");
+  // the compiled network's header, every size and offset a constant
+  constexpr int W = sizeof(BlobHeader) / 4;
+  o("struct HeaderWords { int w[%d]; };\nconstexpr HeaderWords kWords = {{", W);
+  const int32_t* wd = reinterpret_cast<const int32_t*>(&h);
+  for (int i = 0; i < W; ++i) o("%s%d", i ? ", " : "", wd[i]);
+  o.raw("}};\n"
+        "struct SDims {\n  const unsigned char* b;\n"
+        "  static constexpr BlobHeader h = __builtin_bit_cast(BlobHeader, kWords);\n"
+        "  static constexpr int n = h.n, N = h.N, R = h.R, sh = h.self_heating, hasE = h.has_E;\n"
+        "  static constexpr double inv_n = 1.0 / h.n;\n"
+        "  template <class T>\n  __device__ __forceinline__ const T* arr(int off) const {\n"
+        "    return reinterpret_cast<const T*>(b + off);\n  }\n};\n\n}  // namespace nb\n\n");
+  o("extern \"C\" __global__ void __launch_bounds__(256, 1) nb_spec_team(nb::BurnParams B) {\n"
+    "  using namespace nb;\n  extern __shared__ __align__(16) unsigned char sm[];\n"
+    "  const int4* src = reinterpret_cast<const int4*>(B.blob);\n"
+    "  for (int i = threadIdx.x; i < %d; i += blockDim.x) reinterpret_cast<int4*>(sm)[i] = src[i];\n"
+    "  __syncthreads();\n"
+    "  const TNet<%d, 0, SDims> t(SDims{sm}, nullptr);\n"
+    "  double* hot = reinterpret_cast<double*>(sm + %d) + (threadIdx.x / %d) * B.smem_warps;\n"
+    "  CWS w = make_cws(SDims::h, hot, hot + %d);\n  coop_claim_loop(t, w, B);\n}\n",
+    h.bytes / 16, threads, h.bytes, threads, h.thot);
+  return o.s;
+}
+
 // ------------------------------------------------------------------ NVRTC
 
 namespace {

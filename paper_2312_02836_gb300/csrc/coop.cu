@@ -87,11 +87,7 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
   const size_t per_team =
       8 * ((size_t)(k.mem == 0 ? net->h.thot : 0) + net->h.tcold);
   size_t need = std::max<size_t>((size_t)blocks * teams * per_team, 256);
-  // the pre-pass runs one zone per lane: enough lanes for every SM (one block
-  // of 128 for all zones took 0.9 s for 262,144 zones of the 48-species
-  // network), at most 64 an SM, since a lane's arrays hold 25 to 120 KB
-  const long long elanes =
-      std::min<long long>((P.Z + 127) / 128 * 128, ((long long)net->sm_count * 64 + 127) / 128 * 128);
+  const long long elanes = nb::prepass_lanes(net, P.Z);
   if (o.schedule == 1)
     need = std::max(need, (size_t)elanes * (size_t)net->h.lane_doubles * sizeof(double));
   int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);

@@ -16,9 +16,11 @@
 // from memory.  The specialised kernel generated per network at run time
 // supplies another with the same arithmetic.
 #pragma once
+#ifndef __CUDACC_RTC__  // the run-time compiler has no system headers
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
+#endif
 
 #include "blob.h"
 #include "expf64.cuh"

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -29,14 +30,16 @@ struct nb_net_s {
   size_t sched_bytes = 0;
   unsigned char* sched_adj = nullptr;   // the adjoint's claim order and sort scratch
   size_t sched_adj_bytes = 0;
-  // network-specialised kernels by storage variant (1..3): 0 not built,
-  // 1 loaded, -1 failed (log kept)
+  // network-specialised kernels by storage variant (1..3) and, from
+  // kSpecTeam on, by lanes per zone (8, 16, 32): 0 not built, 1 loaded,
+  // -1 failed (log kept)
+  static constexpr int kSpecTeam = 4;
   struct Spec {
     int state = 0;
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kern = nullptr;
     std::string log;
-  } spec[4];
+  } spec[kSpecTeam + 3];
   int last_spec = 0;   // variant the last burn ran (0 generic)
   std::mutex mu;
 };
@@ -86,6 +89,14 @@ inline int ensure(void** p, size_t* have, size_t need) {
   }
   *have = need;
   return NB_OK;
+}
+
+// Lanes of a team launch's pre-pass, one zone per lane: enough for every SM
+// (one block of 128 for all zones took 0.9 s for 262,144 zones of the
+// 48-species network), at most 64 an SM, since a lane's arrays hold up to
+// 120 KB
+inline long long prepass_lanes(nb_net net, long long Z) {
+  return std::min<long long>((Z + 127) / 128 * 128, ((long long)net->sm_count * 64 + 127) / 128 * 128);
 }
 
 // Longest-first claim order: h0 of every zone (a pre-pass on `lanes` lanes of

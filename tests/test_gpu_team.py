@@ -70,3 +70,60 @@ def test_adjoint_threads_per_zone_keep_the_bits(name, t_end, K):
             assert torch.equal(x, y[:, :Z])
     for x, y in zip(grads(9, kernel="coop", ws_in_shared=0), full):
         assert torch.equal(x, y[:, :9])
+
+
+@pytest.mark.parametrize("name", ["chain13", "chain13_heat", "chain13_heat_ap",
+                                  "chain13_heat_scr", "chain13_heat_tab", "chain13_literal"])
+def test_generated_teams_give_the_lane_kernels_bits(name):
+    # the generated kernel's team forms (32, 16, 8 lanes a zone, by zones per
+    # SM) against one zone per lane, on both sides of every line of the rule
+    nb, torch, net, t, tol, sm = _setup(name, 6300, 1e-6)
+    kw = lambda n: dict(zeta=t["zeta"][:n].contiguous()) if "zeta" in t else {}
+    ref = nb.burn(net, *_first(t, 6300), *tol, specialize="generic", **kw(6300))
+    assert net.info()["last_specialized"] == 0
+    for Z in (1, 33, 5 * sm, 5 * sm + 1, 12 * sm, 12 * sm + 1, 40 * sm, 40 * sm + 1):
+        out = nb.burn(net, *_first(t, Z), *tol, **kw(Z))
+        assert net.info()["last_specialized"] > 0
+        _same(torch, out, ref, Z)
+
+
+def test_generated_teams_with_options_tape_and_watchdog():
+    nb, torch, net, t, tol, sm = _setup("chain13_heat", 2 * 160, 1e-6)
+    Z = 320
+    rng = np.random.default_rng(9)
+    lm = torch.from_numpy(rng.normal(0.0, 0.3, (Z, net.R))).cuda()
+    tz = torch.from_numpy(1e-6 * rng.uniform(0.0, 1.0, Z)).cuda()
+    tz[3] = 0.0
+    outs, grads = [], []
+    for sp in ("generic", 0):
+        tape = nb.Tape(net, Z, 900)
+        outs.append(nb.burn(net, *_first(t, Z), tz, tol[1], tol[2], lm, tape=tape, specialize=sp))
+        gY = torch.ones((1, Z, net.N), dtype=torch.float64, device="cuda")
+        grads.append(nb.adjoint(net, tape, gY))
+    _same(torch, outs[0], outs[1], Z)
+    for a, b in zip(*grads):
+        assert torch.equal(a, b)
+    out = nb.burn(net, *_first(t, Z), *tol, max_attempts=20)
+    ref = nb.burn(net, *_first(t, Z), *tol, max_attempts=20, specialize="generic")
+    _same(torch, out, ref, Z)
+    assert int((out.status == 1).sum()) > 0
+    out = nb.burn(net, *_first(t, Z), 1e-3, tol[1], tol[2], time_budget_s=1e-9)
+    assert int((out.status == 6).sum()) == Z
+
+
+def test_last_zones_move_between_warps_with_the_same_bits():
+    # a block's last zones are packed into fewer warps, with and without more
+    # zones than lanes
+    nb, torch, net, t, tol, sm = _setup("chain13_heat", 70000, 1e-7)
+    ref = nb.burn(net, *_first(t, 70000), *tol, kernel="plain")
+    for tpb, bps, n in ((256, 1, 70000), (64, 2, 30011), (160, 1, 5003)):
+        out = nb.burn(net, *_first(t, n), *tol, specialize=3, threads_per_block=tpb,
+                      blocks_per_sm=bps, schedule="fifo")
+        _same(torch, out, ref, n)
+    fixed = nb.Network(gen.network("chain13"))
+    z = gen.zones("chain13", 3000)
+    a = [torch.from_numpy(z[k]).cuda() for k in ("Y", "T9", "rho")]
+    ref = nb.burn(fixed, *a, 1e-6, 1e-8, 1e-12, kernel="plain")
+    for v in (1, 2, 3):
+        out = nb.burn(fixed, *a, 1e-6, 1e-8, 1e-12, specialize=v, threads_per_block=256)
+        _same(torch, out, ref, 3000)
