@@ -18,9 +18,9 @@
 // in blocks of the tape's stride, last block first, recomputes each block's
 // states forward from its checkpointed history window with the forward's
 // own step computation (attempt_solve, so the same bits), then reverses it.
-// One lane per zone (k_adjoint), or one warp per zone for large networks
+// One lane per zone (k_adjoint), or a team of threads per zone
 // (k_adjoint_coop: the same per-zone code with the network spread over the
-// warp, coop.cuh); K cotangent sets share each LU factorisation.
+// team, coop.cuh); K cotangent sets share each LU factorisation.
 #include <cuda_runtime.h>
 #include <cub/device/device_radix_sort.cuh>
 
@@ -108,7 +108,7 @@ struct CoopAdj {
 };
 
 template <int P, int S, int TPB, int MINB>
-__global__ void __launch_bounds__(TPB, MINB) 
+__global__ void __launch_bounds__(TPB, MINB)
     k_adjoint_coop(const __grid_constant__ AdjParams A, const __grid_constant__ CoopAdj C,
                    const __grid_constant__ BlobHeader H) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(TPB, MINB)
     hot = reinterpret_cast<double*>(rest + team_scratch_bytes(P)) + (size_t)tib * C.stride;
     cold = A.ws + team * tcold;
   } else {
-    hot = A.ws + team * (thot + C.a.total + tcold);
-    cold = hot + thot + C.a.total;
+    hot = A.ws + team * (C.stride + tcold);
+    cold = hot + C.stride;
   }
   CWS w = make_cws(H, hot, cold);
   const TAWS a = make_taws(C.a, hot + thot);
@@ -250,6 +250,19 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
   const size_t scratch = team_scratch_bytes(64);
   auto team_fn = &k_adjoint_coop<64, 32, 64, 4>;
   size_t per_unit;   // global workspace per lane (lane kernel) or team (coop)
+  // A lane-recorded tape by teams in the lane order, the lane kernel's bits.
+  // One lane takes 540 ms for its longest zone's reverse sweep whatever the
+  // number of zones up to an SM's lanes (self-heating chain, K = 1); with 8,
+  // 16, 32 lanes a zone 256 zones take 158, 130, 67 ms; 1,024 (7 an SM) 127,
+  // 96, 79; 4,096 (27) 156, 150, 233; 12,000 (79) 241, 354, 605. A large
+  // network's zone keeps two warps busy (48 species, 96 zones, K = 2: 6,971
+  // ms by lanes, 175 ms). A launch shape asked for is the lane kernel's.
+  int lane_team = 0;
+  if (kernel == NB_KERNEL_PERSISTENT && o.threads_per_block <= 0 && o.blocks_per_sm <= 0) {
+    const long long sm = net->sm_count;
+    lane_team = n >= 24 ? 64 : Z <= 12 * sm ? 32 : Z <= 24 * sm ? 16 : Z <= 160 * sm ? 8 : 0;
+  }
+  int teams = 1;   // zones of a block of teams
   if (kernel == NB_KERNEL_COOP) {
     // per team in shared memory: the forward hot arrays and the adjoint's
     const int S = 32;
@@ -293,6 +306,32 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
     const size_t need = (size_t)blocks * per_unit;
     int rc = nb::ensure((void**)&net->ws_adj, &net->ws_adj_bytes, std::max<size_t>(need, 256));
+    if (rc) return rc;
+  } else if (lane_team) {
+    team_layout(h, K, tp->dev.stride, 0, &C.a);
+    C.stride = (h.thot + C.a.total + 7) / 16 * 16 + 8;
+    const size_t team_b = (size_t)C.stride * sizeof(double);
+    const long long per_sm = (Z + net->sm_count - 1) / net->sm_count;
+    tpb = (int)std::max<long long>(lane_team, std::min<long long>(128, (per_sm * lane_team + 31) / 32 * 32));
+    in_smem = blob_b <= 32 * 1024;
+    const size_t fixed = (in_smem ? blob_b : 0) + scratch;
+    while (tpb > lane_team && tpb > 32 && fixed + tpb / lane_team * team_b > net->smem_optin) tpb -= 32;
+    teams = tpb / lane_team;
+    C.smem = fixed + teams * team_b <= net->smem_optin;
+    dyn = fixed + (C.smem ? teams * team_b : 0);
+    team_fn = lane_team == 8    ? &k_adjoint_coop<8, 0, 128, 2>
+              : lane_team == 16 ? &k_adjoint_coop<16, 0, 128, 2>
+              : lane_team == 32 ? &k_adjoint_coop<32, 0, 128, 2>
+                                : &k_adjoint_coop<64, 0, 64, 4>;
+    CK(cudaFuncSetAttribute((const void*)team_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)dyn));
+    int occ = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
+    if (occ < 1) return NB_E_TOO_LARGE;
+    blocks = std::min((long long)occ * net->sm_count, (Z + teams - 1) / teams);
+    per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
+    int rc = nb::ensure((void**)&net->ws_adj, &net->ws_adj_bytes,
+                        std::max<size_t>((size_t)blocks * teams * per_unit, 256));
     if (rc) return rc;
   } else {
     // one zone per lane; smaller blocks when there are few zones per SM
@@ -341,7 +380,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     A.order = i_out;
   }
   CK(cudaMemsetAsync(A.queue, 0, sizeof(unsigned long long), st));
-  if (kernel == NB_KERNEL_COOP)
+  if (kernel == NB_KERNEL_COOP || lane_team)
     team_fn<<<(unsigned)blocks, tpb, dyn, st>>>(A, C, h);
   else
     k_adjoint<<<(unsigned)blocks, tpb, dyn, st>>>(A);

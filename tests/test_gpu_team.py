@@ -127,3 +127,25 @@ def test_last_zones_move_between_warps_with_the_same_bits():
     for v in (1, 2, 3):
         out = nb.burn(fixed, *a, 1e-6, 1e-8, 1e-12, specialize=v, threads_per_block=256)
         _same(torch, out, ref, 3000)
+
+
+@pytest.mark.parametrize("name,K,t_end,big", [("chain13_heat", 2, 1e-6, 4000),
+                                              ("chain13", 1, 1e-6, 25000),
+                                              ("chain13_heat_tab", 9, 1e-6, 400),
+                                              ("net48_adjoint", 2, 1e-5, 70)])
+def test_lane_tapes_by_teams_give_the_lane_adjoints_bits(name, K, t_end, big):
+    # a launch shape asked for runs the lane kernel; without one the teams'
+    # lanes follow the zones per SM
+    nb, torch, net, t, tol, sm = _setup(name, big, t_end)
+    rng = np.random.default_rng(5)
+    for Z in sorted({Z for Z in (1, 33, 12 * sm, 12 * sm + 1, 24 * sm + 1, big) if Z <= big}):
+        lm = torch.from_numpy(rng.normal(0.0, 0.1, net.R)).cuda()
+        tape = nb.Tape(net, Z, 1000)
+        out = nb.burn(net, *_first(t, Z), *tol, lm, tape=tape)
+        assert int((out.status == 0).sum()) == Z
+        gY = torch.from_numpy(rng.normal(size=(K, Z, net.N))).cuda()
+        gE = torch.from_numpy(rng.normal(size=(K, Z))).cuda()
+        gT = torch.from_numpy(rng.normal(size=(K, Z))).cuda()
+        ref = nb.adjoint(net, tape, gY, gE, gT, kernel="persistent", threads_per_block=32)
+        for a, b in zip(nb.adjoint(net, tape, gY, gE, gT), ref):
+            assert torch.equal(a, b)
