@@ -6,9 +6,10 @@
 // NB_MULTI_MAX_SETS (network, zones) sets and runs them in one persistent
 // launch: all lanes of the GPU claim from one device queue that spans every
 // set's zones, so a set of few expensive zones and a set of many cheap ones
-// keep the same warps busy.  Each lane reads the compiled network of the
-// zone it claimed (from global memory, through L1) and runs the generic
-// integrator, so every zone gives the same bits as a single-network burn.
+// keep the same warps busy.  Each lane (or, with few zones or a large
+// network, each team of lanes) reads the compiled network of the zone it
+// claimed and runs the generic integrator, so every zone gives the same bits
+// as a single-network burn.
 #include <cuda_runtime.h>
 #include <cub/device/device_segmented_radix_sort.cuh>
 
@@ -19,6 +20,7 @@
 #include <vector>
 
 #include "blob.h"
+#include "coop.cuh"
 #include "device.cuh"
 #include "host.h"
 #include "../../include/netburn.h"
@@ -98,6 +100,79 @@ __global__ void __launch_bounds__(128, 1) k_burn_multi(const __grid_constant__ M
         zone_finish(t, s, w, P);
         active = false;
       }
+    }
+  }
+}
+
+// The same queue served by teams of P threads in the lane order (coop.cuh),
+// which gives the same bits.  A team's arrays are in shared memory, sized for
+// the largest network (f0 and the history too when cold_smem); the compiled
+// networks are copied there when they all fit.
+struct MultiTeams {
+  MultiParams M;
+  BlobHeader H[NB_MULTI_MAX_SETS];
+  int blob_at[NB_MULTI_MAX_SETS];   // byte offset in shared memory, or -1
+  int blob_bytes;                   // of all the copies
+  int stride;                       // doubles from one team's arrays to the next
+  int cold_smem, cold_doubles;
+};
+
+template <int P>
+__global__ void __launch_bounds__(128, 2) k_multi_team(const __grid_constant__ MultiTeams T) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const MultiParams& M = T.M;
+  for (int m = 0; m < M.n; ++m) {
+    if (T.blob_at[m] < 0) continue;
+    const int4* src = reinterpret_cast<const int4*>(M.p[m].blob);
+    int4* dst = reinterpret_cast<int4*>(sm + T.blob_at[m]);
+    for (int i = threadIdx.x; i < T.H[m].bytes / 16; i += blockDim.x) dst[i] = src[i];
+  }
+  __syncthreads();
+  const int tib = threadIdx.x / P;
+  const long long team = (long long)blockIdx.x * (blockDim.x / P) + tib;
+  double* hot = reinterpret_cast<double*>(sm + T.blob_bytes) + (size_t)tib * T.stride;
+  double* cold = M.ws + team * T.cold_doubles;
+  const unsigned long long total = (unsigned long long)M.off[M.n];
+  const unsigned long long t_start = M.budget_ns ? gpu_ns() : 0ull;
+  const bool lead = threadIdx.x % P == 0;
+  const unsigned mask =
+      P >= 32 ? 0xffffffffu : ((1u << (P & 31)) - 1u) << (threadIdx.x & 31 & ~(P - 1));
+  Zone s;
+  int m = 0;
+  bool active = false;
+  for (;;) {
+    if (!active) {
+      unsigned long long c = 0;
+      if (lead) c = atomicAdd(M.queue, 1ull);
+      c = __shfl_sync(mask, c, 0, P);
+      if (c >= total) break;
+      // the order keeps every position within its own set's range
+      const long long ci = M.order ? (long long)M.order[c] : (long long)c;
+      m = 0;
+      while (m + 1 < M.n && ci >= M.off[m + 1]) ++m;
+      s.z = ci - M.off[m];
+    }
+    const BurnParams& B = M.p[m];
+    const BlobHeader& H = T.H[m];
+    const TNet<P, 0> t(BlobDims(T.blob_at[m] < 0 ? B.blob : sm + T.blob_at[m], H), nullptr);
+    CWS w = make_cws(H, hot, T.cold_smem ? hot + H.thot : cold);
+    bool expired = false;
+    if (M.budget_ns) expired = t.bcast(lead ? gpu_ns() : 0ull) - t_start > M.budget_ns;
+    bool done;
+    if (expired) {
+      if (!active) {
+        zone_timeout_unstarted(t, s.z, B);
+        continue;
+      }
+      s.status = NB_Z_TIMEOUT;
+      done = true;
+    } else {
+      done = active ? zone_attempt(t, s, w, B) : zone_init(t, s, w, B);
+    }
+    active = !done;
+    if (done) {
+      zone_finish(t, s, w, B);
+      t.sync();
     }
   }
 }
@@ -197,7 +272,64 @@ extern "C" int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_e
   const int bps = std::max(1, std::min(o.blocks_per_sm > 0 ? o.blocks_per_sm : 1, occ));
   long long blocks = (long long)bps * host->sm_count;
   blocks = std::min(blocks, (total + tpb - 1) / tpb);
-  const size_t need = (size_t)blocks * tpb * lane_doubles * sizeof(double);
+  // Lanes per zone, 0 for the lane kernel above, which takes 236 to 260 ms for
+  // three chain networks of any 64 to 4,000 zones each (its longest zone):
+  // 3 x 64 zones take 44 ms with 32 lanes, 3 x 500 (10 an SM) 59 ms with 16;
+  // with 8 lanes an SM does a zone in 2 ms, so the two meet near 100 an SM.
+  // With a large network a warp per zone: one lane takes 2.4 s for a zone of
+  // 48 species (4,096 chain and 512 such zones 2,750 ms, by teams 168 ms).
+  // A launch shape asked for is the lane kernel's.
+  const long long sm = host->sm_count;
+  int P = 0;
+  if (o.threads_per_block <= 0 && o.blocks_per_sm <= 0) {
+    P = total <= 5 * sm ? 32 : total <= 12 * sm ? 16 : total <= 100 * sm ? 8 : 0;
+    for (int k = 0; k < n_sets; ++k)
+      if (sets[k].net->h.n >= 24 && sets[k].Z > 0) P = 32;
+  }
+  MultiTeams T;
+  int t_threads = 0;
+  long long t_blocks = 0;
+  size_t t_dyn = 0, t_ws = 0;
+  auto t_fn = P == 8 ? &k_multi_team<8> : P == 16 ? &k_multi_team<16> : &k_multi_team<32>;
+  if (P) {
+    std::memset(&T, 0, sizeof(T));
+    int hot = 0, all = 0, cold = 0, bytes = 0;
+    for (int k = 0; k < n_sets; ++k) {
+      const BlobHeader& h = sets[ord[k]].net->h;
+      T.H[k] = h;
+      hot = std::max(hot, h.thot);
+      cold = std::max(cold, h.tcold);
+      all = std::max(all, h.thot + h.tcold);
+      T.blob_at[k] = bytes;
+      bytes += h.bytes;
+    }
+    const bool copy = bytes <= 48 * 1024;
+    for (int k = 0; k < n_sets && !copy; ++k) T.blob_at[k] = -1;
+    T.blob_bytes = copy ? bytes : 0;
+    T.cold_smem = all <= 1024;
+    T.cold_doubles = T.cold_smem ? 0 : cold;
+    T.stride = ((T.cold_smem ? all : hot) + 7) / 16 * 16 + 8;
+    const size_t team_b = (size_t)T.stride * sizeof(double);
+    const long long per_sm = (total + sm - 1) / sm;
+    t_threads = (int)std::min<long long>(128, (per_sm * P + 31) / 32 * 32);
+    while (t_threads > 32 && T.blob_bytes + t_threads / P * team_b > host->smem_optin) t_threads -= 32;
+    t_dyn = T.blob_bytes + t_threads / P * team_b;
+    int t_occ = 0;
+    if (t_dyn <= host->smem_optin) {
+      CK(cudaFuncSetAttribute((const void*)t_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_dyn));
+      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t_occ, (const void*)t_fn, t_threads, t_dyn));
+    }
+    if (t_occ < 1) {
+      P = 0;   // a zone's arrays don't fit: the lane kernel
+    } else {
+      const int teams = t_threads / P;
+      t_blocks = std::min((long long)t_occ * sm, (total + teams - 1) / teams);
+      t_ws = (size_t)t_blocks * teams * T.cold_doubles * sizeof(double);
+    }
+  }
+  if (P) blocks = std::min(blocks, (nb::prepass_lanes(host, total) + tpb - 1) / tpb);   // of the pre-pass
+  const size_t need =
+      std::max(t_ws, (size_t)blocks * tpb * lane_doubles * sizeof(double));
   int rc = nb::ensure((void**)&host->ws, &host->ws_bytes, need);
   if (rc) return rc;
   M.ws = host->ws;
@@ -231,7 +363,12 @@ extern "C" int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_e
     M.order = i_out;
   }
   CK(cudaMemsetAsync(host->queue, 0, sizeof(unsigned long long), st));
-  k_burn_multi<<<(unsigned)blocks, tpb, 0, st>>>(M);
+  if (P) {
+    T.M = M;
+    t_fn<<<(unsigned)t_blocks, t_threads, t_dyn, st>>>(T);
+  } else {
+    k_burn_multi<<<(unsigned)blocks, tpb, 0, st>>>(M);
+  }
   CK(cudaGetLastError());
   return NB_OK;
 }
