@@ -522,6 +522,11 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
     net->last_spec = spec_variant;
     return NB_OK;
   }
+  if (!specialize_auto_ok(net->h) && net->h.n >= 24 && o.threads_per_block <= 0 &&
+      o.blocks_per_sm <= 0 && o.ws_in_shared <= 0) {
+    int rc = NB_OK;
+    if (nb::launch_lane_teams(net, P, o, st, &rc)) return rc;
+  }
   const size_t blob_b = (size_t)net->h.bytes;
   const size_t hot_warp = (size_t)net->h.hot_doubles * WS_LANES * sizeof(double);
   const int wpb = tpb / 32;

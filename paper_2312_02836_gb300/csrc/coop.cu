@@ -5,7 +5,7 @@
 #include <algorithm>
 
 #include "blob.h"
-#include "coop.cuh"
+#include "coop_kernel.cuh"
 #include "host.h"
 #include "../../include/netburn.h"
 
@@ -13,59 +13,25 @@ using namespace nb;
 
 namespace {
 
-// One zone per team of P threads (coop.cuh), sums of pattern S.  MEM 0: the
-// team's arrays in the global workspace; 1: its Newton-loop arrays in shared
-// memory, f0 and the history in the workspace.  B.smem_warps holds the doubles
-// between one team's arrays and the next in shared memory.
-template <int P, int S, int MEM, int TPB, int MINB>
-__global__ void __launch_bounds__(TPB, MINB) k_burn_coop(const __grid_constant__ BurnParams B, const __grid_constant__ BlobHeader H) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  const unsigned char* blob = B.blob;
-  if (B.blob_in_smem) {
-    const int4* src = reinterpret_cast<const int4*>(B.blob);
-    int4* dst = reinterpret_cast<int4*>(sm);
-    for (int i = threadIdx.x; i < B.blob_bytes / 16; i += blockDim.x) dst[i] = src[i];
-    __syncthreads();
-    blob = sm;
-  }
-  unsigned char* rest = sm + (B.blob_in_smem ? B.blob_bytes : 0);
-  const TNet<P, S> t(BlobDims(blob, H), reinterpret_cast<unsigned long long*>(rest));
-  double* smd = reinterpret_cast<double*>(rest + team_scratch_bytes(P));
-  const int tib = threadIdx.x / P;
-  const long long team = (long long)blockIdx.x * (blockDim.x / P) + tib;
-  const int thot = H.thot, tcold = H.tcold;
-  CWS w;
-  if constexpr (MEM == 1) {
-    w = make_cws(H, smd + (size_t)tib * B.smem_warps, B.ws + team * tcold);
-  } else {
-    double* hot = B.ws + team * (thot + tcold);
-    w = make_cws(H, hot, hot + thot);
-  }
-  coop_claim_loop(t, w, B);
-}
-
-// One built form of the kernel.
-struct TeamKernel {
-  int P, S, mem;
-  void (*fn)(const BurnParams, const BlobHeader);
-};
-#define NB_TEAM(P, S, MEM, TPB, MINB) {P, S, MEM, k_burn_coop<P, S, MEM, TPB, MINB>}
-// All take the registers they want (254): a 168-register form for three
-// blocks of four warps per SM, which the earlier kernel gained from, spills
-// and ran 1030 ms where this one, with two blocks, takes 936 ms (48 species,
-// 65,536 zones).
+// All forms take the registers they want (254): a 168-register form for
+// three blocks of four warps per SM, which the earlier kernel gained from,
+// spills and ran 1030 ms where this one, with two blocks, takes 936 ms (48
+// species, 65,536 zones).
 const TeamKernel kTeamKernels[] = {
-    NB_TEAM(32, 32, 0, 256, 1),   NB_TEAM(32, 32, 1, 256, 1),   NB_TEAM(64, 32, 1, 64, 4),
-    NB_TEAM(128, 32, 1, 128, 2),  NB_TEAM(64, 64, 0, 64, 1),    NB_TEAM(64, 64, 1, 64, 1),
-    NB_TEAM(256, 64, 1, 256, 1),  NB_TEAM(128, 128, 0, 128, 1), NB_TEAM(128, 128, 1, 128, 1),
-    NB_TEAM(256, 128, 1, 256, 1),
+    NB_TEAM(32, 32, 0, 256, 1),
+    NB_TEAM(32, 32, 1, 256, 1),
+    NB_TEAM(64, 32, 1, 64, 4),
+    NB_TEAM(128, 32, 1, 128, 2),
 };
-#undef NB_TEAM
 
 const TeamKernel& team_kernel(int P, int S, int mem) {
   const TeamKernel* hit = kTeamKernels;
   for (const TeamKernel& k : kTeamKernels)
     if (k.P == P && k.S == S && k.mem == mem) hit = &k;
+  for (int i = 0; i < nb::kOtherTeams; ++i) {
+    const TeamKernel& k = nb::kOtherTeamKernels[i];
+    if (k.P == P && k.S == S && k.mem == mem) hit = &k;
+  }
   return *hit;
 }
 
@@ -162,4 +128,21 @@ int nb::launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t
   }
   return launch_team(net, P, o, team_kernel(T, S, hot_smem ? 1 : 0), threads, o.blocks_per_sm,
                      in_smem, st);
+}
+
+// A persistent burn of a large network without a generated kernel by teams in
+// the lane order, the generic lane kernel's bits: one lane takes 2.7 ms a
+// step attempt of the 48-species network and its lanes' arrays leave L2
+// (16,384 zones 3,940 ms, 328 ms by teams).  False when a zone's arrays don't
+// fit in shared memory.
+bool nb::launch_lane_teams(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st, int* rc) {
+  const size_t hot_team = (size_t)net->h.thot * sizeof(double);
+  const size_t scratch = team_scratch_bytes(64);
+  if (hot_team + scratch > net->smem_optin) return false;
+  const bool wide = net->h.nD >= 1024 * net->h.n || P.Z <= 6LL * net->sm_count;
+  int threads = 128;
+  if (!wide)
+    while (threads > 32 && scratch + threads / 32 * hot_team > net->smem_optin) threads -= 32;
+  *rc = launch_team(net, P, o, team_kernel(wide ? 128 : 32, 0, 1), threads, 0, 0, st);
+  return true;
 }

@@ -105,4 +105,7 @@ inline long long prepass_lanes(nb_net net, long long Z) {
 int schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaStream_t st);
 // The cooperative launch (coop.cu).  Caller holds net->mu.
 int launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st);
+// A persistent burn by teams with the lane kernel's bits; false when the
+// network is too large for it (coop.cu).  Caller holds net->mu.
+bool launch_lane_teams(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st, int* rc);
 }  // namespace nb

@@ -149,3 +149,34 @@ def test_lane_tapes_by_teams_give_the_lane_adjoints_bits(name, K, t_end, big):
         ref = nb.adjoint(net, tape, gY, gE, gT, kernel="persistent", threads_per_block=32)
         for a, b in zip(nb.adjoint(net, tape, gY, gE, gT), ref):
             assert torch.equal(a, b)
+
+
+def test_several_networks_by_teams_give_single_burns_bits():
+    # the lanes per zone follow all sets' zones; with a large network a warp
+    nb, torch, _, t, tol, sm = _setup("chain13_heat", 6000, 1e-7)
+    nets = [nb.Network(gen.network(n)) for n in ("chain13_heat", "chain13", "chain13_heat_ap")]
+    lanes = dict(threads_per_block=64, specialize="generic")
+
+    def check(sets):
+        for d, out in zip(sets, nb.burn_multi(sets, *tol)):
+            ref = nb.burn(d["net"], d["Y0"], d["T9"], d["rho"], *tol, **lanes)
+            _same(torch, out, ref, d["Y0"].shape[0])
+
+    def chain(net, n):
+        return dict(zip(("Y0", "T9", "rho"), _first(t, n)), net=net)
+
+    for Z in (1, 5 * sm // 3 + 1, 12 * sm // 3 + 1):
+        check([chain(n, Z) for n in nets])
+    check([chain(n, 5600) for n in nets])     # beyond 100 zones an SM: the lane kernel
+    big, z, _ = gen.problem("net48", 40)
+    a = {k: torch.from_numpy(z[q]).cuda() for k, q in (("Y0", "Y"), ("T9", "T9"), ("rho", "rho"))}
+    check([chain(nets[0], 100), dict(a, net=nb.Network(big))])
+
+
+@pytest.mark.parametrize("name,Z,t_end", [("net48", 1, 1e-5), ("net48", 1000, 1e-6),
+                                          ("net128_heat", 33, 1e-8)])
+def test_large_networks_by_lane_order_teams_give_the_lane_kernels_bits(name, Z, t_end):
+    nb, torch, net, t, tol, sm = _setup(name, Z, t_end)
+    ref = nb.burn(net, *_first(t, Z), *tol, threads_per_block=32)
+    for kw in (dict(), dict(specialize="generic"), dict(schedule="fifo")):
+        _same(torch, nb.burn(net, *_first(t, Z), *tol, **kw), ref, Z)
