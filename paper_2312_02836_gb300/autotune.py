@@ -17,9 +17,12 @@ and where their work arrays live:
 * ``threads_per_block`` and ``blocks_per_sm``: zones in flight.  Fewer lanes
   than zones let the device queue refill lanes whose zone finished; more
   lanes hide more latency but grow the workspace beyond L2;
-* ``kernel="coop"`` (networks of 24 or more state entries): one warp per
-  zone with its Newton-loop arrays in shared memory; threads_per_block sets
-  the warps per block, hence the zones per SM that share its memory.
+* ``kernel="coop"`` (networks of 24 or more state entries): a warp or more
+  per zone with its Newton-loop arrays in shared memory; threads_per_block
+  sets the zones per block, hence those that share an SM's memory.
+
+Without ``threads_per_block`` and ``blocks_per_sm`` the library chooses: few
+zones get several lanes each.  That choice is a candidate too.
 
 Each candidate burns the caller's zones once and is timed with CUDA events
 on the current stream; the fastest wins.  Results are cached per network,
@@ -41,22 +44,19 @@ GENERIC_CANDIDATES = (
 
 SPECIALIZED_CANDIDATES = tuple(
     dict(specialize=v, threads_per_block=tpb, blocks_per_sm=bps)
-    for v in (1, 2, 3) for tpb, bps in ((64, 1), (128, 1), (128, 2), (256, 1)))
+    for v in (1, 2, 3) for tpb, bps in ((64, 1), (128, 1), (128, 2), (256, 1))) + (
+    dict(specialize=0),)
 
 # one warp per zone, its Newton-loop arrays in shared memory (large networks)
 COOP_CANDIDATES = (
     dict(kernel="coop", threads_per_block=0, blocks_per_sm=0),
     dict(kernel="coop", threads_per_block=64, blocks_per_sm=0),
     dict(kernel="coop", threads_per_block=32, blocks_per_sm=0),
-    # one block of four warps per SM: less shared memory taken, more L1 left
-    # for the network's index lists
+    # one block of four warps per SM
     dict(kernel="coop", threads_per_block=128, blocks_per_sm=1),
-    # three blocks of four warps per SM (registers capped, some spilled),
-    # where their shared-memory arrays fit
+    # as many blocks of four warps as fit
     dict(kernel="coop", threads_per_block=128, blocks_per_sm=3),
-    # the same claiming zones in index order: with many zones per warp the
-    # longest-first pre-pass costs more than it saves (48 species: 6.94 s
-    # against 7.80 s at 262,144 zones, 0.60 s against 0.53 s at 16,384)
+    # the same claiming zones in index order, without the pre-pass
     dict(kernel="coop", threads_per_block=128, blocks_per_sm=3, schedule="fifo"),
     # a block of two or four warps per zone: more lanes on each zone's LU
     # where the arrays of one zone take much of an SM's shared memory

@@ -94,21 +94,8 @@ struct BlobHeader {
   int32_t o_tab_t9;     // double [tab_nt] T9 nodes
   int32_t o_tab_lnl;    // double [n_tab * tab_nd * tab_nt] ln lambda at the nodes
   int32_t o_charge;     // double [N] species charges
-  // column-oriented triangular solves (one zone spread over a warp)
-  int32_t o_perm;       // int16 [n] original index of position k
-  int32_t o_ltgt;       // int16 [nL] original row index of each L entry (lslot order)
-  int32_t o_ucol_ptr;   // int32 [n+1] entries of U column k (rows above k)
-  int32_t o_ucol_s;     // int16 [...] their slots
-  int32_t o_ucol_t;     // int16 [...] their original row indices
-  int32_t n_ucol;
-  // transposed solves of the adjoint, column by column
-  int32_t o_utgt;       // int16 [nU] original column index of each U entry (uslot order)
-  int32_t o_lrow_ptr;   // int32 [n+1] entries of L row k (columns left of k)
-  int32_t o_lrow_s;     // int16 [...] their slots
-  int32_t o_lrow_t;     // int16 [...] their original column indices
   int32_t o_dej_ptr;    // int32 [n+1] derivative terms taken by species j
   int32_t o_dej_d;      // int16 [nd] those terms, in increasing order
-  int32_t n_lrow, pad3_;
   // programs of a team of threads that owns one zone (coop.cuh), all in
   // position (elimination) order.  A column program's entry is slot |
   // (2 row + parity) << 16: column k's update of `row`; parity is that of the

@@ -23,6 +23,7 @@
 #include "blob.h"
 #include "codegen.h"
 #include "device.cuh"
+#include "host.h"
 #include "../../include/netburn.h"
 
 namespace nb {
@@ -69,40 +70,50 @@ __global__ void __launch_bounds__(256, 1) k_burn_persistent(BurnParams P) {
   burn_claim_loop(t, w, P);
 }
 
-// Scheduling pre-pass: each zone's starting step h0 (the integrator's own
-// start-up, nothing recorded) as its sort key; zones that finish in start-up
-// go last.
-__global__ void __launch_bounds__(128, 2) k_burn_estimate(BurnParams P, double* key,
-                                                           int32_t* idx) {
-  const Net t = make_net(P.blob);
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const WS w = make_ws(t, P.ws + warp * (long long)t.lane_doubles * WS_LANES + lane);
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x; z < P.Z; z += stride) {
-    Zone s;
-    s.z = z;
-    const bool done = zone_init(t, s, w, P);
-    key[z] = done ? 1e300 : s.h;
-    idx[z] = (int32_t)z;
-  }
+// The arrays the integrator's start-up touches, start_doubles of them per
+// lane: x, f, iw, f0, the first history point, k, rr.  A fifth of a lane's
+// full layout on the 48-species network, so that many lanes fit.
+__device__ __forceinline__ WS make_ws_start(const Net& t, double* base) {
+  WS w = make_ws(t, base);
+  w.x.p = base;
+  w.f.p = base + t.n * WS_LANES;
+  w.iw.p = base + 2 * t.n * WS_LANES;
+  w.f0.p = base + 3 * t.n * WS_LANES;
+  w.xh.p = base + 4 * t.n * WS_LANES;
+  w.k.p = base + 5 * t.n * WS_LANES;
+  w.rr.p = w.k.p + t.R * WS_LANES;
+  w.th.p = w.rr.p + t.R * WS_LANES;
+  w.eh.p = w.th.p + WS_LANES;
+  return w;
 }
 
-// Predicted cost of every zone, (1 + ln(t_end / h0))^2 from the starting step
-// h0 of the integrator's start-up (0 for zones that finish in start-up): on
-// the 48-species network it follows the step attempts with correlation 0.96.
-__global__ void __launch_bounds__(128, 2) k_zone_cost(BurnParams P, double* cost) {
+// Start-up of every zone (the integrator's own, nothing recorded), for its
+// starting step h0.  cost null: h0 as the zone's sort key, zones that finish
+// in start-up last.  Else the predicted cost (1 + ln(t_end / h0))^2 (0 for
+// those zones): on the 48-species network it follows the step attempts with
+// correlation 0.96.  Bound by the latency of the network's lists and of the
+// lanes' arrays, so four blocks per SM at 128 registers: 262,144 zones of 48
+// species take 4.65 ms, with two blocks of 255 registers 5.58, with three
+// 5.06 (its FP64 instructions take 2.9).
+__global__ void __launch_bounds__(128, 4) k_burn_start(BurnParams P, double* key, int32_t* idx,
+                                                       double* cost) {
   const Net t = make_net(P.blob);
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const WS w = make_ws(t, P.ws + warp * (long long)t.lane_doubles * WS_LANES + lane);
+  const long long doubles = nb::start_doubles(t.n, t.R);
+  const WS w = make_ws_start(t, P.ws + warp * doubles * WS_LANES + lane);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x; z < P.Z; z += stride) {
     Zone s;
     s.z = z;
     const bool done = zone_init(t, s, w, P);
-    const double e = done ? -1.0 : log(s.tend / s.h);
-    cost[z] = done ? 0.0 : (1.0 + fmax(e, 0.0)) * (1.0 + fmax(e, 0.0));
+    if (cost) {
+      const double e = done ? -1.0 : log(s.tend / s.h);
+      cost[z] = done ? 0.0 : (1.0 + fmax(e, 0.0)) * (1.0 + fmax(e, 0.0));
+    } else {
+      key[z] = done ? 1e300 : s.h;
+      idx[z] = (int32_t)z;
+    }
   }
 }
 
@@ -132,8 +143,6 @@ __global__ void __launch_bounds__(128, 2) k_burn_plain(BurnParams P) {
 }
 
 // ------------------------------------------------------------------ host side
-
-#include "host.h"
 
 extern "C" {
 
@@ -263,7 +272,7 @@ static int spec_get(nb_net net, int variant, const void** fn) {
     std::vector<char> cubin;
     const bool team = variant >= nb_net_s::kSpecTeam;
     const std::string src =
-        team ? specialized_team_source(net->blob, 8 << (variant - nb_net_s::kSpecTeam))
+        team ? specialized_team_source(net->blob, 4 << (variant - nb_net_s::kSpecTeam))
              : specialized_source(net->blob, variant);
     const char* name = team ? "nb_spec_team" : "nb_spec_burn";
     int rc = compile_specialized(src, &cubin, &sp.log, false);
@@ -338,7 +347,7 @@ extern "C" int nb_specialize_compile(const nb_topology* T, const double* coeffs,
 
 // Longest-first claim order: h0 of every zone (pre-pass over the workspace
 // lanes already allocated), then a radix sort of (h0, zone).  Sets P.order.
-int nb::schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaStream_t st) {
+int nb::schedule_longest_first(nb_net net, BurnParams& P, cudaStream_t st) {
   const long long Z = P.Z;
   if (Z > 0x7fffffffLL) return NB_E_TOO_LARGE;
   size_t temp = 0;
@@ -358,9 +367,10 @@ int nb::schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaS
   void* tmp = base + 2 * kb + 2 * ib;
   BurnParams E = P;
   E.use_tape = 0;
-  const long long fit = (long long)(net->ws_bytes / ((size_t)net->h.lane_doubles * sizeof(double)));
-  const long long eblocks = std::max(1LL, std::min(lanes, fit) / 128);
-  k_burn_estimate<<<(unsigned)eblocks, 128, 0, st>>>(E, k_in, i_in);
+  const long long lane_b = (long long)nb::start_doubles(net->h.n, net->h.R) * 8;
+  const long long lanes =
+      std::min(nb::prepass_lanes(net, Z), (long long)(net->ws_bytes / lane_b) / 128 * 128);
+  k_burn_start<<<(unsigned)std::max(1LL, lanes / 128), 128, 0, st>>>(E, k_in, i_in, nullptr);
   CK(cudaGetLastError());
   CK(cub::DeviceRadixSort::SortPairs(tmp, temp, k_in, k_out, i_in, i_out, (int)Z, 0, 64, st));
   P.order = i_out;
@@ -373,20 +383,29 @@ int nb::schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaS
 // take 94 ms with one lane each, 47, 39, 36 ms with 8, 16, 32. A team costs
 // an SM more instructions per zone, though, so the more zones the fewer
 // lanes: 500 zones 99 / 49 / 41 / 38 ms; 1,500 (10 an SM) 100 / 50 / 44 /
-// 67; 4,096 (27) 100 / 59 / 92 / 144; 8,192 (54) 101 / 116 / 160 / 267. The
-// fixed-temperature, tabulated and effective-rate chains cross between 38
-// and 60 an SM. A launch shape asked for is a lane kernel's.
+// 67; 4,096 (27) 100 / 59 / 92 / 144. With 4 lanes 4,096 zones take 70 ms,
+// 8,192 (54) 83 where 8 lanes take 110 and one 101, 12,345 (81) 136 and 102;
+// effective rates, whose attempt is more rates, which spread: 10,007 (66) 146
+// and 158, 14,000 (92) 178 and 159. At fixed temperature an attempt is mostly
+// what doesn't spread, and 4 lanes never win (8,192 zones 54, 68, 53 ms with
+// 4, 8 and one). A launch shape asked for is a lane kernel's.
 static int spec_team_lanes(nb_net net, const BurnParams& P, const nb_options& o) {
   if (o.threads_per_block > 0 || o.blocks_per_sm > 0) return 0;
   const long long sm = net->sm_count;
-  return P.Z <= 5 * sm ? 32 : P.Z <= 12 * sm ? 16 : P.Z <= 40 * sm ? 8 : 0;
+  const bool sh = net->h.self_heating != 0;
+  const long long four = !sh ? 0 : net->h.n_ap > 0 ? 72 : 60;
+  return P.Z <= 5 * sm                ? 32
+         : P.Z <= 12 * sm             ? 16
+         : P.Z <= (sh ? 35 : 40) * sm ? 8
+         : P.Z <= four * sm           ? 4
+                                      : 0;
 }
 
-// Burn few zones of a network with a generated kernel on its team form (8, 16
-// or 32 lanes a zone); false when it can't be built or doesn't fit.
+// Burn few zones of a network with a generated kernel on its team form (4, 8,
+// 16 or 32 lanes a zone); false when it can't be built or doesn't fit.
 static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int lanes,
                              cudaStream_t st, int* rc) {
-  const int idx = nb_net_s::kSpecTeam + (lanes == 8 ? 0 : lanes == 16 ? 1 : 2);
+  const int idx = nb_net_s::kSpecTeam + (lanes == 4 ? 0 : lanes == 8 ? 1 : lanes == 16 ? 2 : 3);
   // doubles between teams: 8 mod 16, so that two teams' like accesses fall in
   // different halves of the shared-memory banks
   const int stride = (net->h.thot + net->h.tcold + 7) / 16 * 16 + 8;
@@ -406,16 +425,14 @@ static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int
   const int teams = threads / lanes;
   const long long blocks =
       std::min<long long>((long long)occ * net->sm_count, (P.Z + teams - 1) / teams);
-  const long long elanes = nb::prepass_lanes(net, P.Z);
-  *rc = nb::ensure((void**)&net->ws, &net->ws_bytes,
-                   (size_t)elanes * net->h.lane_doubles * sizeof(double));
+  *rc = nb::ensure((void**)&net->ws, &net->ws_bytes, nb::prepass_bytes(net, P.Z));
   if (*rc) return true;
   P.ws = net->ws;
   P.queue = net->queue;
   P.smem_warps = stride;
   P.order = nullptr;
   if (o.schedule == 1 && P.Z > blocks * teams) {   // else every zone starts at once
-    *rc = nb::schedule_longest_first(net, P, elanes, st);
+    *rc = nb::schedule_longest_first(net, P, st);
     if (*rc) return true;
   }
   void* args[] = {&P};
@@ -513,7 +530,7 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
     P.smem_warps = 0;
     P.order = nullptr;
     if (o.schedule == 1 && P.Z > 1) {
-      rc = nb::schedule_longest_first(net, P, blocks * (long long)tpb, st);
+      rc = nb::schedule_longest_first(net, P, st);
       if (rc) return rc;
     }
     CK(cudaMemsetAsync(net->queue, 0, sizeof(unsigned long long), st));
@@ -560,7 +577,7 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
   P.smem_warps = smem_warps;
   P.order = nullptr;
   if (o.schedule == 1 && P.Z > 1) {
-    rc = nb::schedule_longest_first(net, P, blocks * (long long)tpb, st);
+    rc = nb::schedule_longest_first(net, P, st);
     if (rc) return rc;
   }
   CK(cudaMemsetAsync(net->queue, 0, sizeof(unsigned long long), st));
@@ -590,12 +607,11 @@ extern "C" int nb_zone_costs(nb_net net, int64_t Z, const double* Y0, const doub
   P.blob_bytes = net->h.bytes;
   cudaStream_t st = (cudaStream_t)stream;
   std::lock_guard<std::mutex> lk(net->mu);
-  const size_t lane_bytes = (size_t)net->h.lane_doubles * sizeof(double);
-  const long long lanes = std::min<long long>((long long)net->sm_count * 256, (Z + 31) / 32 * 32);
-  int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, (size_t)lanes * lane_bytes);
+  int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, nb::prepass_bytes(net, Z));
   if (rc) return rc;
   P.ws = net->ws;
-  k_zone_cost<<<(unsigned)((lanes + 127) / 128), 128, 0, st>>>(P, cost);
+  k_burn_start<<<(unsigned)(nb::prepass_lanes(net, Z) / 128), 128, 0, st>>>(P, nullptr, nullptr,
+                                                                         cost);
   CK(cudaGetLastError());
   return NB_OK;
 }

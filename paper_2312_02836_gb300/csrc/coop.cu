@@ -53,9 +53,7 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
   const size_t per_team =
       8 * ((size_t)(k.mem == 0 ? net->h.thot : 0) + net->h.tcold);
   size_t need = std::max<size_t>((size_t)blocks * teams * per_team, 256);
-  const long long elanes = nb::prepass_lanes(net, P.Z);
-  if (o.schedule == 1)
-    need = std::max(need, (size_t)elanes * (size_t)net->h.lane_doubles * sizeof(double));
+  if (o.schedule == 1) need = std::max(need, nb::prepass_bytes(net, P.Z));
   int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);
   if (rc) return rc;
   P.ws = net->ws;
@@ -64,7 +62,7 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
   P.smem_warps = stride;
   P.order = nullptr;
   if (o.schedule == 1 && P.Z > 1) {
-    rc = nb::schedule_longest_first(net, P, elanes, st);
+    rc = nb::schedule_longest_first(net, P, st);
     if (rc) return rc;
   }
   CK(cudaMemsetAsync(net->queue, 0, sizeof(unsigned long long), st));

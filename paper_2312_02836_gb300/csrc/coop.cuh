@@ -64,18 +64,31 @@ struct TNet : D_ {
   int lane;        // 0 .. P-1
   unsigned mask;   // the team's lanes in this warp
   unsigned long long* slot;   // P > 32: broadcast slot in shared memory
-  double ser[4];   // this lane's row of g_series
+  // Per-point values (history times, weights, powers of T9) sit one per lane,
+  // or two where the team has fewer than 8 lanes: point j in slot j / SW of
+  // lane j % SW
+  static constexpr int NP = P_ < 8 ? 8 / P_ : 1;
+  double ser[NP][4];   // this lane's rows of g_series
 
   __device__ __forceinline__ TNet(const D_& d, unsigned long long* bslot) : D_(d), slot(bslot) {
     lane = threadIdx.x % P;
     mask = P >= 32 ? 0xffffffffu : ((1u << (P & 31)) - 1u) << (threadIdx.x & 31 & ~(P - 1));
-    const int row = (lane & 31) < 6 ? (lane & 31) : 0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) ser[c] = g_series[row][c];
+    for (int r = 0; r < NP; ++r) {
+      const int row = point(r) < 6 ? point(r) : 0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) ser[r][c] = g_series[row][c];
+    }
   }
   __device__ __forceinline__ int wl() const { return lane & (SW - 1); }
   __device__ __forceinline__ double shfl(double x, int src) const {
     return __shfl_sync(mask, x, src, SW);
+  }
+  // the point in this lane's slot r, and point m's value in every lane
+  __device__ __forceinline__ int point(int r) const { return wl() + SW * r; }
+  __device__ __forceinline__ double pick(const double (&v)[NP], int m) const {
+    if constexpr (NP == 1) return shfl(v[0], m);
+    else return shfl(m < SW ? v[0] : v[1], m & (SW - 1));
   }
   // sum of f over i < cnt: acc <- f(i, acc).  sum1: the lane kernel's single
   // chain, sum2: its two interleaved partial sums; the same in team order.
@@ -229,17 +242,21 @@ __device__ __forceinline__ bool delta_phi_team(const TNet<P, S, D>& t, const TPo
   const double dT = T9 - T9r;
   const double x = dT * r.iT;
   if ((dbits(x) & 0x7fffffffffffffffLL) > 0x3f10000000000000LL) return false;
-  const int l = t.wl();
-  const double pre = l == 0 ? r.iT : l == 1 ? r.it13 : l == 2 ? r.t13 : l == 3 ? r.T53
-                   : l == 4 ? 1.0 : r.hz;
-  const double v = pre * binom4(x, t.ser[0], t.ser[1], t.ser[2], t.ser[3]);
-  d.d1 = t.shfl(v, 0);
-  d.d2 = t.shfl(v, 1);
-  d.d3 = t.shfl(v, 2);
+  double v[TNet<P, S, D>::NP];
+#pragma unroll
+  for (int q = 0; q < TNet<P, S, D>::NP; ++q) {
+    const int l = t.point(q);
+    const double pre = l == 0 ? r.iT : l == 1 ? r.it13 : l == 2 ? r.t13 : l == 3 ? r.T53
+                     : l == 4 ? 1.0 : r.hz;
+    v[q] = pre * binom4(x, t.ser[q][0], t.ser[q][1], t.ser[q][2], t.ser[q][3]);
+  }
+  d.d1 = t.pick(v, 0);
+  d.d2 = t.pick(v, 1);
+  d.d3 = t.pick(v, 2);
   d.d4 = dT;
-  d.d5 = t.shfl(v, 3);
-  d.d6 = t.shfl(v, 4);
-  d.d7 = t.shfl(v, 5);
+  d.d5 = t.pick(v, 3);
+  d.d6 = t.pick(v, 4);
+  d.d7 = t.pick(v, 5);
   return true;
 }
 
@@ -692,29 +709,33 @@ __device__ __forceinline__ const double* solve_M(const TNet<P, S, D>& t, const C
 
 // ---------------------------------------------------------------- step pieces
 
-// alpha_0 in every thread, alpha_j in the threads of lane j of each warp
+// alpha_0 in every thread, alpha_j at point j
 template <int P, int S, class D>
 struct step_alpha<TNet<P, S, D>> {
-  double a0, aj;
+  using T = TNet<P, S, D>;
+  double a0, aj[T::NP];
   unsigned mask;
   __device__ __forceinline__ double operator[](int j) const {
-    return j == 0 ? a0 : __shfl_sync(mask, aj, j, TNet<P, S, D>::SW);
+    if (j == 0) return a0;
+    if constexpr (T::NP == 1) return __shfl_sync(mask, aj[0], j, T::SW);
+    else return __shfl_sync(mask, j < T::SW ? aj[0] : aj[1], j & (T::SW - 1), T::SW);
   }
 };
 
-// out_i = sum_{j<cnt} c_j xh[history j0 + j], c_j held by lane j + c0
+// out_i = sum_{j<cnt} c_j xh[history j0 + j], c_j held by point j + c0
 template <int P, int S, class D, class OUT>
 __device__ __forceinline__ void team_combine(const TNet<P, S, D>& t, const Zone& s, const CWS& w,
-                                             int cnt, int j0, double c, int c0, int beg, int step,
+                                             int cnt, int j0,
+                                             const double (&c)[TNet<P, S, D>::NP], int c0,
                                              OUT out) {
   double cj[KMAX + 1];
   int base[KMAX + 1];
 #pragma unroll
   for (int j = 0; j <= KMAX; ++j) {
-    cj[j] = t.shfl(c, j + c0);
+    cj[j] = t.pick(c, j + c0);
     base[j] = hslot(s, j0 + j < HMAX ? j0 + j : 0) * t.n;
   }
-  for (int i = beg; i < t.n; i += step) {
+  for (int i = t.lane; i < t.n; i += P) {
     double acc = 0.0;
 #pragma unroll
     for (int j = 0; j <= KMAX; ++j)
@@ -723,65 +744,91 @@ __device__ __forceinline__ void team_combine(const TNet<P, S, D>& t, const Zone&
   }
 }
 
-// bdf_alpha, lane j forming alpha_j from its own time tj (t_new in lane 0 and
-// in idle lanes): the team spends one coefficient's instructions instead of k
+// bdf_alpha, point j's lane forming alpha_j from its time tj (t_new at point
+// 0 and at idle ones): the team spends one coefficient's instructions instead
+// of k
 template <int P, int S, class D>
-__device__ __forceinline__ void team_alpha(const TNet<P, S, D>& t, int kk, double t_new, double tj,
-                                           double h, step_alpha<TNet<P, S, D>>& alpha) {
-  const int l = t.wl();
-  const bool mine = l >= 1 && l <= kk;
-  const double ej = t_new - tj;
-  const double rj = 1.0 / (mine ? ej : 1.0);
+__device__ __forceinline__ void team_alpha(const TNet<P, S, D>& t, int kk, double t_new,
+                                           const double (&tj)[TNet<P, S, D>::NP], double h,
+                                           step_alpha<TNet<P, S, D>>& alpha) {
+  constexpr int NP = TNet<P, S, D>::NP;
+  double ej[NP], rj[NP], num[NP], den[NP];
+#pragma unroll
+  for (int r = 0; r < NP; ++r) {
+    const bool mine = t.point(r) >= 1 && t.point(r) <= kk;
+    ej[r] = t_new - tj[r];
+    rj[r] = 1.0 / (mine ? ej[r] : 1.0);
+    num[r] = den[r] = 1.0;
+  }
   double acc = 0.0;
-  for (int m = 1; m <= kk; ++m) acc += t.shfl(rj, m);
-  double num = 1.0, den = 1.0;
+  for (int m = 1; m <= kk; ++m) acc += t.pick(rj, m);
   for (int m = 0; m <= kk; ++m) {
-    const double em = t.shfl(ej, m), tm = t.shfl(tj, m);
-    if (m != l) {
-      if (m != 0) num *= em;
-      den *= tj - tm;
-    }
+    const double em = t.pick(ej, m), tm = t.pick(tj, m);
+#pragma unroll
+    for (int r = 0; r < NP; ++r)
+      if (m != t.point(r)) {
+        if (m != 0) num[r] *= em;
+        den[r] *= tj[r] - tm;
+      }
   }
   alpha.mask = t.mask;
   alpha.a0 = h * acc;
-  alpha.aj = h * num / (mine ? den : 1.0);
+#pragma unroll
+  for (int r = 0; r < NP; ++r) {
+    const bool mine = t.point(r) >= 1 && t.point(r) <= kk;
+    alpha.aj[r] = h * num[r] / (mine ? den[r] : 1.0);
+  }
 }
 
 template <int P, int S, class D>
 __device__ __forceinline__ void step_coeffs(const TNet<P, S, D>& t, const Zone& s, CWS& w,
                                             double atol, double rtol, double h, double t_new,
                                             int kk, step_alpha<TNet<P, S, D>>& alpha) {
-  const int l = t.wl();
-  team_alpha(t, kk, t_new, l >= 1 && l <= kk ? w.th[hslot(s, l - 1)] : t_new, h, alpha);
-  team_combine(t, s, w, kk, 0, alpha.aj, 1, t.lane, P, [&](int i, double a) { w.psi[i] = a; });
+  double tj[TNet<P, S, D>::NP];
+#pragma unroll
+  for (int r = 0; r < TNet<P, S, D>::NP; ++r) {
+    const int l = t.point(r);
+    tj[r] = l >= 1 && l <= kk ? w.th[hslot(s, l - 1)] : t_new;
+  }
+  team_alpha(t, kk, t_new, tj, h, alpha);
+  team_combine(t, s, w, kk, 0, alpha.aj, 1, [&](int i, double a) { w.psi[i] = a; });
   const int b0 = hslot(s, 0) * t.n;
   for (int i = t.lane; i < t.n; i += P) w.iw[i] = recip1(atol + rtol * fabs(w.xh[b0 + i]));
 }
 
-// lane j's Lagrange weight at tt over history j0..j0+q (lagrange_weights)
+// the Lagrange weights at tt over history j0..j0+q (lagrange_weights), one
+// per point
 template <int P, int S, class D>
-__device__ __forceinline__ double team_lagrange(const TNet<P, S, D>& t, const Zone& s, const CWS& w,
-                                                int j0, int q, double tt) {
-  const int l = t.wl();
-  const bool mine = l <= q;
-  const double tj = w.th[hslot(s, mine ? j0 + l : j0)];
-  const double ej = tt - tj;
-  double num = 1.0, den = 1.0;
-  for (int m = 0; m <= q; ++m) {
-    const double em = t.shfl(ej, m), tm = t.shfl(tj, m);
-    if (m != l) {
-      num *= em;
-      den *= tj - tm;
-    }
+__device__ __forceinline__ void team_lagrange(const TNet<P, S, D>& t, const Zone& s, const CWS& w,
+                                              int j0, int q, double tt,
+                                              double (&lw)[TNet<P, S, D>::NP]) {
+  constexpr int NP = TNet<P, S, D>::NP;
+  double tj[NP], ej[NP], num[NP], den[NP];
+#pragma unroll
+  for (int r = 0; r < NP; ++r) {
+    tj[r] = w.th[hslot(s, t.point(r) <= q ? j0 + t.point(r) : j0)];
+    ej[r] = tt - tj[r];
+    num[r] = den[r] = 1.0;
   }
-  return num / (mine ? den : 1.0);
+  for (int m = 0; m <= q; ++m) {
+    const double em = t.pick(ej, m), tm = t.pick(tj, m);
+#pragma unroll
+    for (int r = 0; r < NP; ++r)
+      if (m != t.point(r)) {
+        num[r] *= em;
+        den[r] *= tj[r] - tm;
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < NP; ++r) lw[r] = num[r] / (t.point(r) <= q ? den[r] : 1.0);
 }
 
 template <int P, int S, class D>
 __device__ __forceinline__ void predict(const TNet<P, S, D>& t, const Zone& s, CWS& w, int q,
                                         double t_new) {
-  const double lw = team_lagrange(t, s, w, 0, q, t_new);
-  team_combine(t, s, w, q + 1, 0, lw, 0, t.lane, P, [&](int i, double a) { w.xp[i] = a; });
+  double lw[TNet<P, S, D>::NP];
+  team_lagrange(t, s, w, 0, q, t_new, lw);
+  team_combine(t, s, w, q + 1, 0, lw, 0, [&](int i, double a) { w.xp[i] = a; });
 }
 
 template <int P, int S, class D>
@@ -844,14 +891,15 @@ template <int P, int S, class D>
 __device__ __forceinline__ double order_estimate(const TNet<P, S, D>& t, const Zone& s, CWS& w,
                                                  int q, double h) {
   const double t0 = w.th[hslot(s, 0)];
-  const double lw = team_lagrange(t, s, w, 1, q, t0);
+  double lw[TNet<P, S, D>::NP];
+  team_lagrange(t, s, w, 1, q, t0, lw);
   const double c = h / (t0 - w.th[hslot(s, q + 1)]);
   const int b0 = hslot(s, 0) * t.n;
   double cj[KMAX + 1];
   int base[KMAX + 1];
 #pragma unroll
   for (int j = 0; j <= KMAX; ++j) {
-    cj[j] = t.shfl(lw, j);
+    cj[j] = t.pick(lw, j);
     base[j] = hslot(s, j + 1) * t.n;
   }
   return team_square(t, w, [&](int i) {

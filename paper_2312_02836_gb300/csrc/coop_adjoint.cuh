@@ -113,9 +113,14 @@ template <int P, int S, class D>
 __device__ __forceinline__ void adj_alpha(const TNet<P, S, D>& t, const AdjParams& A, long long z,
                                           int s, int kk, double h,
                                           step_alpha<TNet<P, S, D>>& alpha) {
-  const int l = t.wl();
   const double t_new = sched_ptr(A, z, s)[0];
-  team_alpha(t, kk, t_new, l >= 1 && l <= kk ? sched_ptr(A, z, s - l)[0] : t_new, h, alpha);
+  double tj[TNet<P, S, D>::NP];
+#pragma unroll
+  for (int r = 0; r < TNet<P, S, D>::NP; ++r) {
+    const int l = t.point(r);
+    tj[r] = l >= 1 && l <= kk ? sched_ptr(A, z, s - l)[0] : t_new;
+  }
+  team_alpha(t, kk, t_new, tj, h, alpha);
 }
 
 template <int P, int S, class D>

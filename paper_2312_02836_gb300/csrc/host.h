@@ -31,7 +31,7 @@ struct nb_net_s {
   unsigned char* sched_adj = nullptr;   // the adjoint's claim order and sort scratch
   size_t sched_adj_bytes = 0;
   // network-specialised kernels by storage variant (1..3) and, from
-  // kSpecTeam on, by lanes per zone (8, 16, 32): 0 not built, 1 loaded,
+  // kSpecTeam on, by lanes per zone (4, 8, 16, 32): 0 not built, 1 loaded,
   // -1 failed (log kept)
   static constexpr int kSpecTeam = 4;
   struct Spec {
@@ -39,7 +39,7 @@ struct nb_net_s {
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kern = nullptr;
     std::string log;
-  } spec[kSpecTeam + 3];
+  } spec[kSpecTeam + 4];
   int last_spec = 0;   // variant the last burn ran (0 generic)
   std::mutex mu;
 };
@@ -91,18 +91,22 @@ inline int ensure(void** p, size_t* have, size_t need) {
   return NB_OK;
 }
 
-// Lanes of a team launch's pre-pass, one zone per lane: enough for every SM
-// (one block of 128 for all zones took 0.9 s for 262,144 zones of the
-// 48-species network), at most 64 an SM, since a lane's arrays hold up to
-// 120 KB
+// doubles per lane of a start-up pass (k_burn_start)
+__host__ __device__ constexpr int start_doubles(int n, int R) { return 5 * n + 2 * R + 2; }
+// its lanes, one zone each at a time: what four blocks per SM hold (one block
+// of 128 lanes for all zones took 0.9 s for 262,144 zones of the 48-species
+// network), and their workspace
 inline long long prepass_lanes(nb_net net, long long Z) {
-  return std::min<long long>((Z + 127) / 128 * 128, ((long long)net->sm_count * 64 + 127) / 128 * 128);
+  return std::min<long long>((Z + 127) / 128 * 128, (long long)net->sm_count * 512);
+}
+inline size_t prepass_bytes(nb_net net, long long Z) {
+  return (size_t)prepass_lanes(net, Z) * start_doubles(net->h.n, net->h.R) * sizeof(double);
 }
 
-// Longest-first claim order: h0 of every zone (a pre-pass on `lanes` lanes of
-// the workspace already allocated), then a radix sort of (h0, zone).  Sets
+// Longest-first claim order: h0 of every zone (a start-up pass in the
+// workspace already allocated), then a radix sort of (h0, zone).  Sets
 // P.order.  (burn.cu)
-int schedule_longest_first(nb_net net, BurnParams& P, long long lanes, cudaStream_t st);
+int schedule_longest_first(nb_net net, BurnParams& P, cudaStream_t st);
 // The cooperative launch (coop.cu).  Caller holds net->mu.
 int launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st);
 // A persistent burn by teams with the lane kernel's bits; false when the

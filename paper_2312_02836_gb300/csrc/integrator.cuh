@@ -25,13 +25,13 @@
 // network held in memory; the specialised one is generated per network as
 // straight-line code with every index a constant and compiled at run time.
 // Both run one zone per lane and perform the same floating-point operations
-// in the same order, so they give the same bits.  The cooperative one
-// (coop.cuh) runs one zone per team of W threads, a warp or a block of two
-// or four warps: its vector loops are spread over the team (vbeg/vstep),
-// its sums are team reductions (vsum) and its phases are separated by the
-// team's barriers (vsync); every thread holds the same copy of the zone's
-// scalars, so control flow stays uniform.  For the one-zone-per-lane types
-// these helpers reduce to the plain loops and do nothing.
+// in the same order, so they give the same bits.  The team one (coop.cuh)
+// runs one zone per team of threads: its vector loops are spread over the
+// team (vbeg/vstep), its phases are separated by the team's barriers (vsync),
+// its sums (vsum1, and the pieces of a step it overloads) are the team's;
+// every thread holds the same copy of the zone's scalars, so control flow
+// stays uniform.  For the one-zone-per-lane types these helpers reduce to the
+// plain loops and do nothing.
 //
 // This header is also compiled by the run-time compiler, so it includes no
 // system header.
@@ -55,7 +55,7 @@
 
 namespace nb {
 
-// Network types that spread one zone over the lanes of a warp specialise this
+// Network types that spread one zone over a team of threads specialise this
 template <class NT>
 struct is_coop {
   static constexpr bool value = false;

@@ -327,7 +327,6 @@ extern "C" int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_e
       t_ws = (size_t)t_blocks * teams * T.cold_doubles * sizeof(double);
     }
   }
-  if (P) blocks = std::min(blocks, (nb::prepass_lanes(host, total) + tpb - 1) / tpb);   // of the pre-pass
   const size_t need =
       std::max(t_ws, (size_t)blocks * tpb * lane_doubles * sizeof(double));
   int rc = nb::ensure((void**)&host->ws, &host->ws_bytes, need);

@@ -201,32 +201,32 @@ int build_blob(const nb_topology* T, const double* coeffs,
         if (F[pi][pj]) at[slot[pi][pj]] = {pi, pj};
     int s = 0;
     for (const auto& e : at) {
-        int i = perm[e.first], j = perm[e.second];
-        uint8_t fl = (i == j) ? SLOT_DIAG : 0;
-        if (i < N && j < N) {
-          for (int r = 0; r < R; ++r) {
-            auto it = stoich[r].find(i);
-            if (it == stoich[r].end()) continue;
-            for (int d : dterms_of_r[r])
-              if (dt_j[d] == j) { js_src.push_back((int16_t)d); js_c.push_back(it->second); }
-          }
-        } else if (i < N && j == N) {
-          for (int r = 0; r < R; ++r) {
-            auto it = stoich[r].find(i);
-            if (it != stoich[r].end()) { js_src.push_back((int16_t)(nd + r)); js_c.push_back(it->second); }
-          }
-        } else if (i == N && j < N) {
-          fl |= SLOT_TROW;
-          for (int r = 0; r < R; ++r)
-            for (int d : dterms_of_r[r])
-              if (dt_j[d] == j) { js_src.push_back((int16_t)d); js_c.push_back(T->Q[r]); }
-        } else {  // (T, T)
-          fl |= SLOT_TT;
-          for (int r = 0; r < R; ++r) { js_src.push_back((int16_t)(nd + r)); js_c.push_back(T->Q[r]); }
+      int i = perm[e.first], j = perm[e.second];
+      uint8_t fl = (i == j) ? SLOT_DIAG : 0;
+      if (i < N && j < N) {
+        for (int r = 0; r < R; ++r) {
+          auto it = stoich[r].find(i);
+          if (it == stoich[r].end()) continue;
+          for (int d : dterms_of_r[r])
+            if (dt_j[d] == j) { js_src.push_back((int16_t)d); js_c.push_back(it->second); }
         }
-        js_flag[s] = fl;
-        js_ptr[++s] = (int32_t)js_src.size();
+      } else if (i < N && j == N) {
+        for (int r = 0; r < R; ++r) {
+          auto it = stoich[r].find(i);
+          if (it != stoich[r].end()) { js_src.push_back((int16_t)(nd + r)); js_c.push_back(it->second); }
+        }
+      } else if (i == N && j < N) {
+        fl |= SLOT_TROW;
+        for (int r = 0; r < R; ++r)
+          for (int d : dterms_of_r[r])
+            if (dt_j[d] == j) { js_src.push_back((int16_t)d); js_c.push_back(T->Q[r]); }
+      } else {  // (T, T)
+        fl |= SLOT_TT;
+        for (int r = 0; r < R; ++r) { js_src.push_back((int16_t)(nd + r)); js_c.push_back(T->Q[r]); }
       }
+      js_flag[s] = fl;
+      js_ptr[++s] = (int32_t)js_src.size();
+    }
   }
 
   // LU program
@@ -279,30 +279,6 @@ int build_blob(const nb_topology* T, const double* coeffs,
   tri(false, true, true, &tbw, &tbw_s, &tbw_c);   // L^T u = v
   std::vector<int32_t> diag_orig(n);
   for (int i = 0; i < n; ++i) diag_orig[i] = slot[pos[i]][pos[i]];
-  // column-oriented solves: rows of the L entries, and U by columns
-  std::vector<int16_t> perm16(n), ltgt, ucol_s, ucol_t;
-  std::vector<int32_t> ucol_ptr(n + 1, 0);
-  for (int k = 0; k < n; ++k) perm16[k] = (int16_t)perm[k];
-  for (int k = 0; k < n; ++k)
-    for (int i = k + 1; i < n; ++i)
-      if (F[i][k]) ltgt.push_back((int16_t)perm[i]);
-  for (int k = 0; k < n; ++k) {
-    for (int i = 0; i < k; ++i)
-      if (F[i][k]) { ucol_s.push_back((int16_t)slot[i][k]); ucol_t.push_back((int16_t)perm[i]); }
-    ucol_ptr[k + 1] = (int32_t)ucol_s.size();
-  }
-  // transposed solves: the columns of the U entries (pivot rows), L by rows
-  std::vector<int16_t> utgt, lrow_s, lrow_t;
-  std::vector<int32_t> lrow_ptr(n + 1, 0);
-  for (int k = 0; k < n; ++k)
-    for (int j = k + 1; j < n; ++j)
-      if (F[k][j]) utgt.push_back((int16_t)perm[j]);
-  for (int k = 0; k < n; ++k) {
-    for (int i = 0; i < k; ++i)
-      if (F[k][i]) { lrow_s.push_back((int16_t)slot[k][i]); lrow_t.push_back((int16_t)perm[i]); }
-    lrow_ptr[k + 1] = (int32_t)lrow_s.size();
-  }
-
   // adjoint: species entries of each rate, d f_i / d p_r = c_ir R_r
   std::vector<int32_t> rg_ptr(R + 1, 0);
   std::vector<int16_t> rg_i;
@@ -422,17 +398,6 @@ int build_blob(const nb_topology* T, const double* coeffs,
   h.o_rg_ptr = B.add(rg_ptr);
   h.o_rg_i = B.add(rg_i);
   h.o_rg_c = B.add(rg_c);
-  h.o_perm = B.add(perm16);
-  h.o_ltgt = B.add(ltgt);
-  h.o_ucol_ptr = B.add(ucol_ptr);
-  h.o_ucol_s = B.add(ucol_s);
-  h.o_ucol_t = B.add(ucol_t);
-  h.n_ucol = (int32_t)ucol_s.size();
-  h.o_utgt = B.add(utgt);
-  h.o_lrow_ptr = B.add(lrow_ptr);
-  h.o_lrow_s = B.add(lrow_s);
-  h.o_lrow_t = B.add(lrow_t);
-  h.n_lrow = (int32_t)lrow_s.size();
   {
     // derivative terms by the species they are taken by (state index j < N)
     std::vector<int32_t> dej_ptr(n + 1, 0);

@@ -75,13 +75,14 @@ def test_adjoint_threads_per_zone_keep_the_bits(name, t_end, K):
 @pytest.mark.parametrize("name", ["chain13", "chain13_heat", "chain13_heat_ap",
                                   "chain13_heat_scr", "chain13_heat_tab", "chain13_literal"])
 def test_generated_teams_give_the_lane_kernels_bits(name):
-    # the generated kernel's team forms (32, 16, 8 lanes a zone, by zones per
+    # the generated kernel's team forms (32, 16, 8, 4 lanes a zone, by zones per
     # SM) against one zone per lane, on both sides of every line of the rule
-    nb, torch, net, t, tol, sm = _setup(name, 6300, 1e-6)
+    nb, torch, net, t, tol, sm = _setup(name, 11600, 1e-6)
     kw = lambda n: dict(zeta=t["zeta"][:n].contiguous()) if "zeta" in t else {}
-    ref = nb.burn(net, *_first(t, 6300), *tol, specialize="generic", **kw(6300))
+    ref = nb.burn(net, *_first(t, 11600), *tol, specialize="generic", **kw(11600))
     assert net.info()["last_specialized"] == 0
-    for Z in (1, 33, 5 * sm, 5 * sm + 1, 12 * sm, 12 * sm + 1, 40 * sm, 40 * sm + 1):
+    for Z in (1, 33, 5 * sm, 5 * sm + 1, 12 * sm, 12 * sm + 1, 35 * sm + 1, 40 * sm + 1, 60 * sm,
+              60 * sm + 1, 72 * sm + 1):
         out = nb.burn(net, *_first(t, Z), *tol, **kw(Z))
         assert net.info()["last_specialized"] > 0
         _same(torch, out, ref, Z)
