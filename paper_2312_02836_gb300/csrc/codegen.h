@@ -18,8 +18,8 @@ bool specialize_auto_ok(const BlobHeader& h);
 // CUDA source of the specialised kernel `nb_spec_burn` for a compiled network.
 std::string specialized_source(const std::vector<uint8_t>& blob, int variant);
 
-// CUDA source of the team form `nb_spec_team`: `threads` (8 or 16) lanes per
-// zone, the lane kernel's bits.
+// CUDA source of the team form `nb_spec_team`: `threads` (4, 8, 16 or
+// 32) lanes per zone, the lane kernel's bits.
 std::string specialized_team_source(const std::vector<uint8_t>& blob, int threads);
 
 // Compile to an sm_103a cubin with the run-time compiler (loaded on first

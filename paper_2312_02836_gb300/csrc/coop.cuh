@@ -1,5 +1,5 @@
-// coop.cuh -- one zone per team of threads: 8 or 16 lanes of a warp, a warp,
-// or a block of two to eight warps.  The network evaluation, the linear
+// coop.cuh -- one zone per team of threads: 4, 8 or 16 lanes of a warp, a
+// warp, or a block of two to eight warps.  The network evaluation, the linear
 // algebra and the per-step scalars of the integrator (integrator.cuh) are
 // spread over the team.
 //

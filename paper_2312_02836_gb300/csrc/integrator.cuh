@@ -160,6 +160,7 @@ struct BurnParams {
   TapeDev tape;
   int use_tape;
   int smem_warps;             // warps per block with hot arrays in shared memory
+                              // (team kernels: doubles from team to team there)
   unsigned long long budget_ns;  // watchdog budget per block, 0 = none
   const int32_t* order;       // claim order (zone index per claim), or null
   const double* t_end_zone;   // [Z] per-zone end time (operator split), or null
