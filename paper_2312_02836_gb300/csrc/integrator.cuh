@@ -1126,7 +1126,7 @@ NB_HD __forceinline__ void zone_finish(const NT& t, const Zone& s, const WT& w,
   }
 }
 
-#ifdef __CUDA_ARCH__
+#if defined(__CUDA_ARCH__) || defined(NB_EMULATED_BLOCK)  // a test runs it on the host
 // The barrier at which a block's warps start their attempts together, and,
 // once the queue is empty, the packing of its last zones.  True when the
 // block has none left.
@@ -1140,14 +1140,18 @@ NB_HD __forceinline__ void zone_finish(const NT& t, const Zone& s, const WT& w,
 //    history is in the workspace, the rest is the Zone struct) and the warp
 //    stops.  Taken first: a warp of the scheduler with the most running
 //    warps, then the one with the fewest zones.
+// A warp whose zones all end at once is at the next turn while another still
+// reads the counts of this one, so the turns alternate between two rows of
+// counts: a row is written again only after the next turn's barrier.
 template <class NT, class WT>
 __device__ __forceinline__ bool block_done(const NT&, WT& w, Zone& s, bool& active,
-                                           bool& retired, bool& fresh) {
-  __shared__ int cnt[8];        // running zones of each warp
+                                           bool& retired, bool& fresh, int turn) {
+  __shared__ int counts[2][8];  // running zones of each warp
   __shared__ Zone moved[32];
   __shared__ int from[32];      // thread | fresh << 16
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const unsigned on = __ballot_sync(0xffffffffu, active), below = (1u << lane) - 1u;
+  int* cnt = counts[turn];
   if (lane == 0) cnt[warp] = __popc(on);
   if (!__syncthreads_or(retired)) return false;
   int total = 0, running = 0, load[4] = {0, 0, 0, 0};
@@ -1183,7 +1187,7 @@ __device__ __forceinline__ bool block_done(const NT&, WT& w, Zone& s, bool& acti
         w.take((long long)((src >> 5) - warp) * NT::lane_doubles * WS_LANES + (src & 31) - lane);
       }
     }
-    __syncthreads();   // cnt, moved and the arrays of the old lanes are free
+    __syncthreads();   // moved and the arrays of the old lanes are free
   }
   return false;
 }
@@ -1202,6 +1206,7 @@ __device__ __forceinline__ void burn_claim_loop(const NT& t, WT& w, const BurnPa
   s.h = s.t = s.tend = 0.0;
   s.k = s.nh = 1;
   bool active = false, retired = false, fresh = false;
+  [[maybe_unused]] int turn = 0;
   const unsigned long long t_start = P.budget_ns ? gpu_ns() : 0ull;
   for (;;) {
     const unsigned need = __ballot_sync(0xffffffffu, !active && !retired);
@@ -1222,7 +1227,7 @@ __device__ __forceinline__ void burn_claim_loop(const NT& t, WT& w, const BurnPa
       }
     }
     if constexpr (in_step<NT>::value) {
-      if (block_done(t, w, s, active, retired, fresh)) break;
+      if (block_done(t, w, s, active, retired, fresh, turn ^= 1)) break;
     } else {
       if (__all_sync(0xffffffffu, retired)) break;
     }

@@ -181,3 +181,16 @@ def test_large_networks_by_lane_order_teams_give_the_lane_kernels_bits(name, Z, 
     ref = nb.burn(net, *_first(t, Z), *tol, threads_per_block=32)
     for kw in (dict(), dict(specialize="generic"), dict(schedule="fifo")):
         _same(torch, nb.burn(net, *_first(t, Z), *tol, **kw), ref, Z)
+
+
+@pytest.mark.parametrize("kw", [dict(max_attempts=1), dict(max_attempts=7),
+                                dict(max_attempts=300)])
+def test_zones_of_a_block_that_end_at_once(kw):
+    # all zones of a warp reach the attempt limit in the same turn, while
+    # other warps' zones end earlier or have ended
+    nb, torch, net, t, tol, sm = _setup("chain13_heat", 20000)
+    ref = nb.burn(net, *_first(t, 20000), *tol, kernel="plain", **kw)
+    assert int((ref.status == 1).sum()) > 0
+    for tpb, n in ((256, 20000), (160, 20000), (64, 700)):
+        out = nb.burn(net, *_first(t, n), *tol, specialize=3, threads_per_block=tpb, **kw)
+        _same(torch, out, ref, n)
