@@ -312,10 +312,13 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     C.stride = (h.thot + C.a.total + 7) / 16 * 16 + 8;
     const size_t team_b = (size_t)C.stride * sizeof(double);
     const long long per_sm = (Z + net->sm_count - 1) / net->sm_count;
-    tpb = (int)std::max<long long>(lane_team, std::min<long long>(128, (per_sm * lane_team + 31) / 32 * 32));
+    // a team of several warps is a block of its own (its barrier and its
+    // broadcasts are the block's)
+    tpb = lane_team > 32 ? lane_team
+                         : (int)std::min<long long>(128, (per_sm * lane_team + 31) / 32 * 32);
     in_smem = blob_b <= 32 * 1024;
     const size_t fixed = (in_smem ? blob_b : 0) + scratch;
-    while (tpb > lane_team && tpb > 32 && fixed + tpb / lane_team * team_b > net->smem_optin) tpb -= 32;
+    while (lane_team <= 32 && tpb > 32 && fixed + tpb / lane_team * team_b > net->smem_optin) tpb -= 32;
     teams = tpb / lane_team;
     C.smem = fixed + teams * team_b <= net->smem_optin;
     dyn = fixed + (C.smem ? teams * team_b : 0);

@@ -194,3 +194,18 @@ def test_zones_of_a_block_that_end_at_once(kw):
     for tpb, n in ((256, 20000), (160, 20000), (64, 700)):
         out = nb.burn(net, *_first(t, n), *tol, specialize=3, threads_per_block=tpb, **kw)
         _same(torch, out, ref, n)
+
+
+@pytest.mark.parametrize("K", [1, 2])
+def test_large_networks_lane_tapes_beyond_a_zone_an_sm(K):
+    # a team of two warps is a block of its own, however many zones an SM gets
+    nb, torch, net, t, tol, sm = _setup("net48_adjoint", 3 * 160 + 1, 1e-6)
+    rng = np.random.default_rng(8)
+    for Z in (sm, sm + 1, 3 * sm):
+        tape = nb.Tape(net, Z, 400)
+        nb.burn(net, *_first(t, Z), *tol, tape=tape)
+        gY = torch.from_numpy(rng.normal(size=(K, Z, net.N))).cuda()
+        gE = torch.from_numpy(rng.normal(size=(K, Z))).cuda()
+        ref = nb.adjoint(net, tape, gY, gE, kernel="persistent", threads_per_block=32)
+        for a, b in zip(nb.adjoint(net, tape, gY, gE), ref):
+            assert torch.equal(a, b)
