@@ -336,7 +336,9 @@ class BurnGraph:
     them in place (same shapes) and call ``replay()``; ``out`` holds the
     results.  Capture happens after one ordinary burn with the same launch
     options, so the device workspace is already allocated and the captured
-    work is one counter reset and one kernel launch."""
+    work is one counter reset and one kernel launch (with the longest-first
+    claim order, its pre-pass and sort before them).  The network keeps the
+    workspace of a capture until it is freed, whatever later calls need."""
 
     def __init__(self, net: "Network", Y0, T9, rho, t_end, rtol, atol,
                  ln_mult=None, **launch):

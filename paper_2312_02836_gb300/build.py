@@ -12,7 +12,7 @@ LIB = os.path.join(BUILD, "libnetburn.so")
 SOURCES = ["burn.cu", "coop.cu", "coop_forms.cu", "adjoint.cu", "noalloc.cu", "multi.cu",
            "expcheck.cu", "netload.cpp", "codegen.cpp"]
 HEADERS = ["blob.h", "device.cuh", "integrator.cuh", "adjoint.cuh", "coop.cuh", "coop_adjoint.cuh",
-           "coop_kernel.cuh", "host.h", "expf64.cuh", "codegen.h"]
+           "coop_kernel.cuh", "devbuf.h", "host.h", "expf64.cuh", "codegen.h"]
 # headers the run-time compiler needs, embedded as text into the library
 # (name as written in the #include directive, path)
 EMBED = [("expf64.cuh", "csrc/expf64.cuh"), ("integrator.cuh", "csrc/integrator.cuh"),

@@ -305,7 +305,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     if (blocks > Z) blocks = Z;
     per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
     const size_t need = (size_t)blocks * per_unit;
-    int rc = nb::ensure((void**)&net->ws_adj, &net->ws_adj_bytes, std::max<size_t>(need, 256));
+    int rc = nb::ensure(net->ws_adj, net->kept, std::max<size_t>(need, 256), st);
     if (rc) return rc;
   } else if (lane_team) {
     team_layout(h, K, tp->dev.stride, 0, &C.a);
@@ -333,8 +333,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     if (occ < 1) return NB_E_TOO_LARGE;
     blocks = std::min((long long)occ * net->sm_count, (Z + teams - 1) / teams);
     per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
-    int rc = nb::ensure((void**)&net->ws_adj, &net->ws_adj_bytes,
-                        std::max<size_t>((size_t)blocks * teams * per_unit, 256));
+    int rc = nb::ensure(net->ws_adj, net->kept, std::max<size_t>((size_t)blocks * teams * per_unit, 256), st);
     if (rc) return rc;
   } else {
     // one zone per lane; smaller blocks when there are few zones per SM
@@ -353,11 +352,11 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     const long long needed = (Z + tpb - 1) / tpb;
     if (blocks > needed) blocks = needed;
     per_unit = (size_t)A.lane_doubles * sizeof(double);
-    int rc = nb::ensure((void**)&net->ws_adj, &net->ws_adj_bytes, (size_t)blocks * tpb * per_unit);
+    int rc = nb::ensure(net->ws_adj, net->kept, (size_t)blocks * tpb * per_unit, st);
     if (rc) return rc;
   }
   int rc = NB_OK;
-  A.ws = net->ws_adj;
+  A.ws = net->ws_adj.p;
   A.queue = net->queue + 1;   // a second counter in the same allocation
   A.blob_in_smem = in_smem;
   // Claim order: the tape holds every zone's step count, the exact length of
@@ -371,14 +370,14 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
                                                  (int32_t*)nullptr, (int)Z, 0, 32, st));
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t ib = al((size_t)Z * 4);
-    rc = nb::ensure((void**)&net->sched_adj, &net->sched_adj_bytes, 3 * ib + al(temp));
+    rc = nb::ensure(net->sched_adj, net->kept, 3 * ib + al(temp), st);
     if (rc) return rc;
-    int32_t* k_out = (int32_t*)net->sched_adj;
-    int32_t* i_in = (int32_t*)(net->sched_adj + ib);
-    int32_t* i_out = (int32_t*)(net->sched_adj + 2 * ib);
+    int32_t* k_out = (int32_t*)net->sched_adj.p;
+    int32_t* i_in = (int32_t*)(net->sched_adj.p + ib);
+    int32_t* i_out = (int32_t*)(net->sched_adj.p + 2 * ib);
     k_zone_index<<<(unsigned)((Z + 255) / 256), 256, 0, st>>>(i_in, Z);
     CK(cudaGetLastError());
-    CK(cub::DeviceRadixSort::SortPairsDescending(net->sched_adj + 3 * ib, temp, tp->dev.steps,
+    CK(cub::DeviceRadixSort::SortPairsDescending(net->sched_adj.p + 3 * ib, temp, tp->dev.steps,
                                                  k_out, i_in, i_out, (int)Z, 0, 32, st));
     A.order = i_out;
   }

@@ -216,11 +216,12 @@ int nb_net_free(nb_net net) {
   if (!net) return NB_E_ARG;
   cudaFree(net->d_blob);
   cudaFree(net->queue);
-  if (net->ws) cudaFree(net->ws);
-  if (net->stage) cudaFree(net->stage);
-  if (net->ws_adj) cudaFree(net->ws_adj);
-  if (net->sched) cudaFree(net->sched);
-  if (net->sched_adj) cudaFree(net->sched_adj);
+  cudaFree(net->ws.p);
+  cudaFree(net->stage.p);
+  cudaFree(net->ws_adj.p);
+  cudaFree(net->sched.p);
+  cudaFree(net->sched_adj.p);
+  for (void* p : net->kept) cudaFree(p);
   for (auto& sp : net->spec)
     if (sp.lib) cudaLibraryUnload(sp.lib);
   delete net;
@@ -357,9 +358,9 @@ int nb::schedule_longest_first(nb_net net, BurnParams& P, cudaStream_t st) {
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t kb = al((size_t)Z * 8), ib = al((size_t)Z * 4);
   const size_t need = 2 * kb + 2 * ib + al(temp);
-  int rc = nb::ensure((void**)&net->sched, &net->sched_bytes, need);
+  int rc = nb::ensure(net->sched, net->kept, need, st);
   if (rc) return rc;
-  unsigned char* base = net->sched;
+  unsigned char* base = net->sched.p;
   double* k_in = (double*)base;
   double* k_out = (double*)(base + kb);
   int32_t* i_in = (int32_t*)(base + 2 * kb);
@@ -369,7 +370,7 @@ int nb::schedule_longest_first(nb_net net, BurnParams& P, cudaStream_t st) {
   E.use_tape = 0;
   const long long lane_b = (long long)nb::start_doubles(net->h.n, net->h.R) * 8;
   const long long lanes =
-      std::min(nb::prepass_lanes(net, Z), (long long)(net->ws_bytes / lane_b) / 128 * 128);
+      std::min(nb::prepass_lanes(net, Z), (long long)(net->ws.bytes / lane_b) / 128 * 128);
   k_burn_start<<<(unsigned)std::max(1LL, lanes / 128), 128, 0, st>>>(E, k_in, i_in, nullptr);
   CK(cudaGetLastError());
   CK(cub::DeviceRadixSort::SortPairs(tmp, temp, k_in, k_out, i_in, i_out, (int)Z, 0, 64, st));
@@ -425,9 +426,9 @@ static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int
   const int teams = threads / lanes;
   const long long blocks =
       std::min<long long>((long long)occ * net->sm_count, (P.Z + teams - 1) / teams);
-  *rc = nb::ensure((void**)&net->ws, &net->ws_bytes, nb::prepass_bytes(net, P.Z));
+  *rc = nb::ensure(net->ws, net->kept, nb::prepass_bytes(net, P.Z), st);
   if (*rc) return true;
-  P.ws = net->ws;
+  P.ws = net->ws.p;
   P.queue = net->queue;
   P.smem_warps = stride;
   P.order = nullptr;
@@ -463,9 +464,9 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
   if (o.kernel == NB_KERNEL_PLAIN) {
     const long long blocks = (P.Z + tpb - 1) / tpb;
     const size_t need = (size_t)blocks * tpb * lane_bytes;
-    int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);
+    int rc = nb::ensure(net->ws, net->kept, need, st);
     if (rc) return rc;
-    P.ws = net->ws;
+    P.ws = net->ws.p;
     P.blob_in_smem = 0;
     k_burn_plain<<<(unsigned)blocks, tpb, 0, st>>>(P);
     CK(cudaGetLastError());
@@ -522,9 +523,9 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
     if (blocks > needed_blocks) blocks = needed_blocks;
     size_t need = std::max<size_t>((size_t)blocks * tpb * lane_bytes, 256);
     if (o.schedule == 1) need = std::max(need, (size_t)128 * lane_bytes);  // pre-pass lanes
-    int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);
+    int rc = nb::ensure(net->ws, net->kept, need, st);
     if (rc) return rc;
-    P.ws = net->ws;
+    P.ws = net->ws.p;
     P.queue = net->queue;
     P.blob_in_smem = 0;
     P.smem_warps = 0;
@@ -569,9 +570,9 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
   const size_t per_block = (size_t)32 * (smem_warps * cold_bytes + (wpb - smem_warps) * lane_bytes);
   size_t need = std::max<size_t>((size_t)blocks * per_block, 256);
   if (o.schedule == 1) need = std::max(need, (size_t)128 * lane_bytes);  // pre-pass lanes
-  int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);
+  int rc = nb::ensure(net->ws, net->kept, need, st);
   if (rc) return rc;
-  P.ws = net->ws;
+  P.ws = net->ws.p;
   P.queue = net->queue;
   P.blob_in_smem = in_smem;
   P.smem_warps = smem_warps;
@@ -607,9 +608,9 @@ extern "C" int nb_zone_costs(nb_net net, int64_t Z, const double* Y0, const doub
   P.blob_bytes = net->h.bytes;
   cudaStream_t st = (cudaStream_t)stream;
   std::lock_guard<std::mutex> lk(net->mu);
-  int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, nb::prepass_bytes(net, Z));
+  int rc = nb::ensure(net->ws, net->kept, nb::prepass_bytes(net, Z), st);
   if (rc) return rc;
-  P.ws = net->ws;
+  P.ws = net->ws.p;
   k_burn_start<<<(unsigned)(nb::prepass_lanes(net, Z) / 128), 128, 0, st>>>(P, nullptr, nullptr,
                                                                          cost);
   CK(cudaGetLastError());
@@ -701,9 +702,9 @@ extern "C" int nb_burn_batch_host(nb_net net, int64_t Z, const double* Y0,
                off_s = off_c + al(z4 * NCOUNT), total = off_s + al(z4);
   cudaStream_t st = (cudaStream_t)stream;
   std::lock_guard<std::mutex> lk(net->mu);
-  rc = nb::ensure((void**)&net->stage, &net->stage_bytes, total);
+  rc = nb::ensure(net->stage, net->kept, total, st);
   if (rc) return rc;
-  unsigned char* b = net->stage;
+  unsigned char* b = net->stage.p;
   CK(cudaMemcpyAsync(b + off_Y0, Y0, zN, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(b + off_T0, T9_0, z8, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(b + off_rho, rho, z8, cudaMemcpyHostToDevice, st));

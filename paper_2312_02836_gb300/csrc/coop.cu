@@ -54,9 +54,9 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
       8 * ((size_t)(k.mem == 0 ? net->h.thot : 0) + net->h.tcold);
   size_t need = std::max<size_t>((size_t)blocks * teams * per_team, 256);
   if (o.schedule == 1) need = std::max(need, nb::prepass_bytes(net, P.Z));
-  int rc = nb::ensure((void**)&net->ws, &net->ws_bytes, need);
+  int rc = nb::ensure(net->ws, net->kept, need, st);
   if (rc) return rc;
-  P.ws = net->ws;
+  P.ws = net->ws.p;
   P.queue = net->queue;
   P.blob_in_smem = in_smem;
   P.smem_warps = stride;

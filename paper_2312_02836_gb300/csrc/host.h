@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "blob.h"
+#include "devbuf.h"
 #include "device.cuh"
 #include "../../include/netburn.h"
 
@@ -18,18 +19,14 @@ struct nb_net_s {
   int device = 0;
   int sm_count = 0;
   size_t smem_optin = 0;
-  double* ws = nullptr;
-  size_t ws_bytes = 0;
+  nb::DevBuf<double> ws;
   unsigned long long* queue = nullptr;
   // staging for the host-pointer entry point
-  unsigned char* stage = nullptr;
-  size_t stage_bytes = 0;
-  double* ws_adj = nullptr;   // adjoint per-lane workspace
-  size_t ws_adj_bytes = 0;
-  unsigned char* sched = nullptr;   // claim-order keys, indices, sort scratch
-  size_t sched_bytes = 0;
-  unsigned char* sched_adj = nullptr;   // the adjoint's claim order and sort scratch
-  size_t sched_adj_bytes = 0;
+  nb::DevBuf<unsigned char> stage;
+  nb::DevBuf<double> ws_adj;              // adjoint per-lane workspace
+  nb::DevBuf<unsigned char> sched;        // claim-order keys, indices, sort scratch
+  nb::DevBuf<unsigned char> sched_adj;    // the adjoint's claim order and sort scratch
+  std::vector<void*> kept;                // outgrown buffers that captured graphs use
   // network-specialised kernels by storage variant (1..3) and, from
   // kSpecTeam on, by lanes per zone (4, 8, 16, 32): 0 not built, 1 loaded,
   // -1 failed (log kept)
@@ -77,20 +74,6 @@ inline void tape_release(nb_tape_s* tp) {
 
 
 namespace nb {
-// (Re)allocate a device buffer of at least `need` bytes.
-inline int ensure(void** p, size_t* have, size_t need) {
-  if (*have >= need && *p) return NB_OK;
-  if (*p) cudaFree(*p);
-  *p = nullptr;
-  *have = 0;
-  if (cudaMalloc(p, need) != cudaSuccess) {
-    *p = nullptr;
-    return NB_E_NOMEM;
-  }
-  *have = need;
-  return NB_OK;
-}
-
 // doubles per lane of a start-up pass (k_burn_start)
 __host__ __device__ constexpr int start_doubles(int n, int R) { return 5 * n + 2 * R + 2; }
 // its lanes, one zone each at a time: what four blocks per SM hold (one block

@@ -329,9 +329,9 @@ extern "C" int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_e
   }
   const size_t need =
       std::max(t_ws, (size_t)blocks * tpb * lane_doubles * sizeof(double));
-  int rc = nb::ensure((void**)&host->ws, &host->ws_bytes, need);
+  int rc = nb::ensure(host->ws, host->kept, need, st);
   if (rc) return rc;
-  M.ws = host->ws;
+  M.ws = host->ws.p;
   M.queue = host->queue;
   M.order = nullptr;
   if (o.schedule == 1 && total > 1 && total <= 0x7fffffffLL) {
@@ -345,9 +345,9 @@ extern "C" int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_e
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t kb = al((size_t)total * 8), ib = al((size_t)total * 4);
     const size_t sb = al(sizeof(seg));
-    rc = nb::ensure((void**)&host->sched, &host->sched_bytes, 2 * kb + 2 * ib + sb + al(temp));
+    rc = nb::ensure(host->sched, host->kept, 2 * kb + 2 * ib + sb + al(temp), st);
     if (rc) return rc;
-    unsigned char* base = host->sched;
+    unsigned char* base = host->sched.p;
     double* k_in = (double*)base;
     double* k_out = (double*)(base + kb);
     int32_t* i_in = (int32_t*)(base + 2 * kb);

@@ -68,3 +68,29 @@ def test_watchdog_ends_zones_with_timeout(kernel):
                     kernel=kernel)
     torch.cuda.synchronize()
     assert torch.equal(again.Y, full.Y)
+
+
+@pytest.mark.parametrize("name,Z,later", [
+    ("net48", 400, dict(threads_per_block=32)),
+    ("chain13_heat", 64, dict(Z=20000)),
+    ("chain13_heat", 5000, dict(specialize="generic"))])
+def test_graph_outlives_larger_calls_on_its_network(name, Z, later):
+    # the later calls need more workspace than the captured burn (and more
+    # room for the claim order), twice
+    nb, torch, net, z, s, t = _setup(name, 40000 if "Z" in later else Z)
+    later = dict(later)
+    big = later.pop("Z", Z)
+    nc = nb.Network(net)
+    tol = (1e-6, s["rtol"], s["atol"])
+    first = lambda n: [t[k][:n].contiguous() for k in ("Y", "T9", "rho")]
+    g = nb.BurnGraph(nc, *first(Z), *tol)
+    ref = [x.clone() for x in g.replay()]
+    other = []
+    for n in (big, 2 * big) if big > Z else (big, big):
+        nb.burn(nc, *first(n), *tol, **later)
+        # what the library gave back would be handed out again here
+        other.append(torch.full((1 << 22,), float("nan"), dtype=torch.float64, device="cuda"))
+        for x in g.out:
+            x.zero_()
+        for a, b in zip(g.replay(), ref):
+            assert torch.equal(a, b)
