@@ -133,10 +133,13 @@ __global__ void __launch_bounds__(128, 2) k_multi_team(const __grid_constant__ M
   double* hot = reinterpret_cast<double*>(sm + T.blob_bytes) + (size_t)tib * T.stride;
   double* cold = M.ws + team * T.cold_doubles;
   const unsigned long long total = (unsigned long long)M.off[M.n];
-  const unsigned long long t_start = M.budget_ns ? gpu_ns() : 0ull;
   const bool lead = threadIdx.x % P == 0;
   const unsigned mask =
       P >= 32 ? 0xffffffffu : ((1u << (P & 31)) - 1u) << (threadIdx.x & 31 & ~(P - 1));
+  // the team's watchdog starts at thread 0's clock and reads it: threads that
+  // each read their own could decide apart, and part at a shuffle
+  unsigned long long t_start = 0ull;
+  if (M.budget_ns) t_start = __shfl_sync(mask, lead ? gpu_ns() : 0ull, 0, P);
   Zone s;
   int m = 0;
   bool active = false;

@@ -133,3 +133,21 @@ def test_multi_network_batch_against_oracle():
         rep = compare(to_numpy(out), o, s["atol"], rtol=s["rtol"], spread=spread)
         assert (to_numpy(out)["status"] == 0).all()
         print(name, rep)
+
+
+@pytest.mark.parametrize("Z", [5, 300, 1200, 4000])
+@pytest.mark.parametrize("budget", [1e-9, 3e-3])
+def test_watchdog_of_several_networks(Z, budget):
+    # few zones (teams of 32, 16, 8 lanes a zone) and the lane kernel: zones
+    # that end in time have a full burn's bits, all others time out
+    nb, torch = _mods()
+    sets = [_set(nb, torch, name, Z)[0]
+            for name in ("chain13_heat", "chain13", "chain13_heat_ap", "chain13_literal")]
+    full = nb.burn_multi(sets, 1e-3, 1e-8, 1e-12)
+    cut = nb.burn_multi(sets, 1e-3, 1e-8, 1e-12, time_budget_s=budget)
+    for a, b in zip(cut, full):
+        ok = a.status == 0
+        assert bool(((a.status == 0) | (a.status == 6)).all())
+        assert torch.equal(a.Y[ok], b.Y[ok]) and torch.equal(a.T9[ok], b.T9[ok])
+        assert bool(torch.isfinite(a.Y).all())
+    assert sum(int((a.status == 6).sum()) for a in cut) > 0
