@@ -103,7 +103,8 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams A) {
 // and its adjoint arrays sit in shared memory after the (optional) blob copy,
 // C.stride doubles per team; else everything is in the workspace.
 struct CoopAdj {
-  int smem, stride;
+  int smem;
+  long long stride;
   TeamAdj a;
 };
 
@@ -165,22 +166,6 @@ __global__ void __launch_bounds__(TPB, MINB)
 __global__ void k_zone_index(int32_t* idx, long long Z) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < Z) idx[i] = (int32_t)i;
-}
-
-// offsets of a team's adjoint arrays for K cotangent sets
-void team_layout(const BlobHeader& h, int K, int stride, int S, TeamAdj* a) {
-  int off = 0;
-  auto take = [&](long long cnt) { const int o = off; off += (int)cnt; return o; };
-  a->lam = take((long long)HMAX * K * h.n);
-  a->ee = take(HMAX * K);
-  a->gr = take((long long)K * h.R);
-  a->gt = take(K);
-  a->mu = take((long long)K * team_mu(h.n, S));
-  a->de = take(h.n);
-  a->seg = take((long long)stride * h.n);
-  a->ce = take(K);
-  a->vs = take(h.self_heating ? 0 : (long long)(S > 0 ? 1 : K) * h.R);
-  a->total = (off + 1) & ~1;
 }
 
 }  // namespace

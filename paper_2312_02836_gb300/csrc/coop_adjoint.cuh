@@ -6,9 +6,11 @@
 
 namespace nb {
 
-// a team's adjoint arrays, offsets in doubles from its first one
+// a team's adjoint arrays, offsets in doubles from its first one (64 bits: a
+// tape's stride may be any number, and the recomputed block has that many
+// states)
 struct TeamAdj {
-  int lam, ee, gr, gt, mu, de, seg, ce, vs, total;
+  long long lam, ee, gr, gt, mu, de, seg, ce, vs, total;
 };
 
 // mu: K solve vectors; ce: e_q h / alpha_0; vs: [K, R] rate terms (lane order
@@ -27,6 +29,22 @@ __device__ __forceinline__ TAWS make_taws(const TeamAdj& A, double* base) {
 
 // doubles of one solve vector
 __host__ __device__ constexpr int team_mu(int n, int S) { return S > 0 ? n : 3 * n; }
+
+// offsets of a team's adjoint arrays for K cotangent sets
+inline void team_layout(const BlobHeader& h, int K, int stride, int S, TeamAdj* a) {
+  long long off = 0;
+  auto take = [&](long long cnt) { const long long o = off; off += cnt; return o; };
+  a->lam = take((long long)HMAX * K * h.n);
+  a->ee = take(HMAX * K);
+  a->gr = take((long long)K * h.R);
+  a->gt = take(K);
+  a->mu = take((long long)K * team_mu(h.n, S));
+  a->de = take(h.n);
+  a->seg = take((long long)stride * h.n);
+  a->ce = take(K);
+  a->vs = take(h.self_heating ? 0 : (long long)(S > 0 ? 1 : K) * h.R);
+  a->total = (off + 1) & ~1LL;
+}
 
 // v_q <- M^-T v_q of K vectors at once, each n (team order) or 3 n (lane
 // order: partial sums, then the solution) doubles from v + q * stride in
