@@ -22,7 +22,7 @@ def run_block(tmp_path_factory):
     if gxx is None:
         pytest.skip("no C++ compiler")
     out = str(tmp_path_factory.mktemp("host") / "libblocktail.so")
-    subprocess.check_call([gxx, "-O1", "-std=c++17", "-shared", "-fPIC",
+    subprocess.check_call([gxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic",
                            "-I", os.path.join(ROOT, "include"),
                            os.path.join(HERE, "host", "block_tail.cpp"), "-o", out])
     fn = C.CDLL(out).run_block

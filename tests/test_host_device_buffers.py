@@ -20,7 +20,9 @@ def buf(tmp_path):
         pytest.skip("no compiler")
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     out = str(tmp_path / "libdevbuf.so")
-    subprocess.check_call([gxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-I", cuda,
+    subprocess.check_call([gxx, "-O1", "-std=c++17", "-shared", "-fPIC",
+                           # the fakes, whatever the process has loaded
+                           "-Wl,-Bsymbolic", "-I", cuda,
                            os.path.join(HERE, "host", "device_buffers.cpp"), "-o", out])
     lib = C.CDLL(out)
     lib.buf_call.argtypes = [C.c_size_t, C.c_int, C.c_int]
