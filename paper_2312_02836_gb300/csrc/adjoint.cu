@@ -280,8 +280,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     in_smem = o.blob_in_shared != 0 && blob_b <= 96 * 1024 &&
               blob_b + scratch + (C.smem ? team_b : 0) <= net->smem_optin;
     dyn = (in_smem ? blob_b : 0) + scratch + (C.smem ? team_b : 0);
-    CK(cudaFuncSetAttribute((const void*)team_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)dyn));
+    CK(nb::allow_shared((const void*)team_fn, net->smem_optin));
     int occ = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
     if (occ < 1) return NB_E_TOO_LARGE;
@@ -311,8 +310,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
               : lane_team == 16 ? &k_adjoint_coop<16, 0, 128, 2>
               : lane_team == 32 ? &k_adjoint_coop<32, 0, 128, 2>
                                 : &k_adjoint_coop<64, 0, 64, 4>;
-    CK(cudaFuncSetAttribute((const void*)team_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)dyn));
+    CK(nb::allow_shared((const void*)team_fn, net->smem_optin));
     int occ = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
     if (occ < 1) return NB_E_TOO_LARGE;
@@ -329,7 +327,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     in_smem = blob_b <= 96 * 1024 ? 1 : 0;
     dyn = in_smem ? blob_b : 0;
     if (dyn > 48 * 1024)
-      CK(cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+      CK(nb::allow_shared((const void*)k_adjoint, net->smem_optin));
     int occ = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_adjoint, tpb, dyn));
     blocks = (long long)std::max(1, std::min(o.blocks_per_sm > 0 ? o.blocks_per_sm : 2, occ)) *

@@ -418,7 +418,7 @@ static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int
   const void* fn = nullptr;
   if (dyn > net->smem_optin || spec_get(net, idx, &fn) != NB_OK) return false;
   int occ = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess ||
+  if (nb::allow_shared(fn, net->smem_optin) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, dyn) != cudaSuccess || occ < 1) {
     cudaGetLastError();
     return false;
@@ -556,7 +556,7 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
   size_t dyn = (in_smem ? blob_b : 0) + (size_t)smem_warps * hot_warp;
   if (dyn > net->smem_optin) return NB_E_TOO_LARGE;
   if (dyn > 48 * 1024)
-    CK(cudaFuncSetAttribute(k_burn_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    CK(nb::allow_shared((const void*)k_burn_persistent, net->smem_optin));
   int bps = o.blocks_per_sm;
   int occ = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_burn_persistent, tpb, dyn));

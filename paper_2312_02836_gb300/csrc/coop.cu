@@ -44,7 +44,7 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
   const int stride = k.mem == 0 ? 0 : net->h.thot;
   const size_t dyn = blob_b + team_scratch_bytes(k.P) + (size_t)teams * stride * sizeof(double);
   if (dyn > net->smem_optin) return NB_E_TOO_LARGE;
-  CK(cudaFuncSetAttribute((const void*)k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  CK(nb::allow_shared((const void*)k.fn, net->smem_optin));
   int occ = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k.fn, threads, dyn));
   if (occ < 1) return NB_E_TOO_LARGE;

@@ -74,6 +74,14 @@ inline void tape_release(nb_tape_s* tp) {
 
 
 namespace nb {
+// Let a kernel be launched with any dynamic shared memory a block may have
+// (smem_optin; the kernels here have no other).  The limit belongs to the
+// kernel, not to a launch: set to one launch's size, another thread's call for
+// a smaller network could lower it before that launch, which would fail.
+inline cudaError_t allow_shared(const void* fn, size_t smem_optin) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_optin);
+}
+
 // doubles per lane of a start-up pass (k_burn_start)
 __host__ __device__ constexpr int start_doubles(int n, int R) { return 5 * n + 2 * R + 2; }
 // its lanes, one zone each at a time: what four blocks per SM hold (one block

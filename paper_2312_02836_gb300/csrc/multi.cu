@@ -319,7 +319,7 @@ extern "C" int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_e
     t_dyn = T.blob_bytes + t_threads / P * team_b;
     int t_occ = 0;
     if (t_dyn <= host->smem_optin) {
-      CK(cudaFuncSetAttribute((const void*)t_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_dyn));
+      CK(nb::allow_shared((const void*)t_fn, host->smem_optin));
       CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t_occ, (const void*)t_fn, t_threads, t_dyn));
     }
     if (t_occ < 1) {

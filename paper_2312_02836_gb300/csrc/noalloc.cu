@@ -107,7 +107,7 @@ extern "C" int nb_burn_batch_noalloc(nb_net net, int64_t Z, const double* Y0,
   const size_t dyn = in_smem ? blob_b : 0;
   if (dyn > net->smem_optin) return NB_E_TOO_LARGE;
   if (dyn > 48 * 1024)
-    CK(cudaFuncSetAttribute(k_burn_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    CK(nb::allow_shared((const void*)k_burn_noalloc, net->smem_optin));
   int occ = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_burn_noalloc, tpb, dyn));
   if (occ < 1) return NB_E_TOO_LARGE;

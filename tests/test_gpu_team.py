@@ -209,3 +209,51 @@ def test_large_networks_lane_tapes_beyond_a_zone_an_sm(K):
         ref = nb.adjoint(net, tape, gY, gE, kernel="persistent", threads_per_block=32)
         for a, b in zip(nb.adjoint(net, tape, gY, gE), ref):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("call", ["burn", "coop", "adjoint", "multi"])
+def test_networks_of_different_sizes_from_two_threads(call):
+    # each thread its own network and stream; the kernels are the same, their
+    # shared memory differs from network to network
+    import threading
+    nb, torch, *_ = _setup("chain13", 1)
+    ref, got, errors = {}, {}, []
+
+    def work(name, Z, rounds, into):
+        _, _, net, t, tol, _ = _setup(name, Z, 1e-12)
+        a = _first(t, Z)
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            stream.wait_stream(torch.cuda.default_stream())
+            for _ in range(rounds):
+                if call == "multi":
+                    out = nb.burn_multi([dict(net=net, Y0=a[0], T9=a[1], rho=a[2])], *tol)[0]
+                elif call == "adjoint":
+                    tape = nb.Tape(net, Z, 50)
+                    nb.burn(net, *a, *tol, tape=tape)
+                    out = nb.adjoint(net, tape, torch.ones((1, Z, net.N), dtype=torch.float64,
+                                                           device="cuda"))
+                else:
+                    out = nb.burn(net, *a, *tol,
+                                  kernel="coop" if call == "coop" else "persistent")
+        stream.synchronize()
+        into[name] = out
+
+    def guarded(*args):
+        try:
+            work(*args)
+        except Exception as e:      # a refused launch
+            errors.append(e)
+
+    pairs = (("net48", 8), ("net128_heat", 8))
+    for name, Z in pairs:
+        work(name, Z, 1, ref)
+    threads = [threading.Thread(target=guarded, args=(name, Z, 400, got)) for name, Z in pairs]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not errors
+    for name, _ in pairs:
+        for a, b in zip(got[name], ref[name]):
+            assert torch.equal(a, b)
