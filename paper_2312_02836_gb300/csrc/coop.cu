@@ -71,6 +71,22 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
   return NB_OK;
 }
 
+// Whether the options' shape fits: a zone's Newton-loop arrays as the lane
+// kernels lay them out, `warps` such zones a block (0: as few as one) or one
+// with the partial sums of wpz warps, and the blob where it is asked for.
+// Teams keep a little more a zone; where that alone is too much, the arrays go
+// to the workspace.
+bool coop_shape_fits(nb_net net, const nb_options& o, int wpz, int warps) {
+  const size_t blob_b = (size_t)net->h.bytes, optin = net->smem_optin;
+  const size_t zone_b = (size_t)net->h.hot_doubles * sizeof(double);
+  const size_t red = wpz > 1 ? (2 * wpz + 1) * sizeof(double) : 0;
+  const bool hot = o.ws_in_shared != 0 && zone_b + red <= optin;
+  const bool blob = o.blob_in_shared >= 0
+                        ? o.blob_in_shared != 0
+                        : blob_b <= 96 * 1024 && blob_b + (hot ? zone_b : 0) + red <= optin;
+  return (blob ? blob_b : 0) + red + (hot ? std::max(warps, 1) * zone_b : 0) <= optin;
+}
+
 }  // namespace
 
 // Sums in team order of S = 32 x warps_per_zone partial sums.
@@ -98,19 +114,18 @@ int nb::launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t
   if (wpz == 1 && o.threads_per_block > 0 &&
       (o.threads_per_block % 32 != 0 || o.threads_per_block > 256))
     return NB_E_ARG;
+  const int warps_asked = wpz == 1 && o.threads_per_block > 0 ? o.threads_per_block / 32 : 0;
+  if (!coop_shape_fits(net, o, wpz, warps_asked)) return NB_E_TOO_LARGE;
   const size_t scratch = team_scratch_bytes(64);
-  const bool hot_smem = o.ws_in_shared != 0 && hot_team + scratch <= net->smem_optin;
+  // a blob asked for in shared memory goes first
+  const size_t blob_asked = o.blob_in_shared > 0 ? blob_b : 0;
+  const bool hot_smem =
+      o.ws_in_shared != 0 && blob_asked + hot_team + scratch <= net->smem_optin;
   int in_smem = o.blob_in_shared;
   if (in_smem < 0)
     in_smem = blob_b <= 96 * 1024 && blob_b + (hot_smem ? hot_team : 0) + scratch <= net->smem_optin;
   const size_t fixed = (in_smem ? blob_b : 0) + scratch;
   const int S = 32 * wpz;
-  // an explicit block of several zones has to fit with one zone per warp
-  const size_t warp_b = (size_t)net->h.hot_doubles * sizeof(double);
-  const int warps_asked = wpz == 1 ? o.threads_per_block / 32 : 0;
-  if (warps_asked > 0 && o.ws_in_shared != 0 && warp_b <= net->smem_optin &&
-      (in_smem ? blob_b : 0) + warps_asked * warp_b > net->smem_optin)
-    return NB_E_TOO_LARGE;
   const bool large = net->h.nD >= 1024 * net->h.n;
   int T = S;
   if (hot_smem) {

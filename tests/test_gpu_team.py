@@ -257,3 +257,35 @@ def test_networks_of_different_sizes_from_two_threads(call):
     for name, _ in pairs:
         for a, b in zip(got[name], ref[name]):
             assert torch.equal(a, b)
+
+
+def test_a_blob_and_a_zone_that_just_fit_shared_memory():
+    # 202,560 bytes of compiled network and 29,808 of one zone's arrays of the
+    # 232,448 a block may have; a team's arrays are 144 bytes more
+    import dataclasses
+    import paper_2312_02836_gb300 as nb
+    import torch
+    from gen import workloads as wl
+    N = 68
+    rng = np.random.Generator(np.random.PCG64(31))
+    reac, prod = wl._random_topology(rng, N, (81, 136, 27))
+    keep = np.arange(reac.shape[0]) != 8
+    spec = dataclasses.replace(gen.network("net48"), N=N, R=int(keep.sum()),
+                               reactants=reac[keep], products=prod[keep],
+                               A=np.arange(1, N + 1, dtype=np.float64),
+                               coeffs=wl._draw_coeffs(rng, reac.shape[0])[keep])
+    net = nb.Network(spec)
+    Z = 40
+    Y = np.zeros((Z, N))
+    Y[:, :4] = gen.zones("net48", Z)["Y"][:, :4]
+    a = [torch.from_numpy(x).cuda() for x in (Y, gen.zones("net48", Z)["T9"],
+                                              gen.zones("net48", Z)["rho"])]
+    tol = (1e-6, 1e-8, 1e-12)
+    ref = nb.burn(net, *a, *tol, kernel="coop")
+    for tpb in (0, 32):
+        out = nb.burn(net, *a, *tol, kernel="coop", blob_in_shared=1, threads_per_block=tpb)
+        _same(torch, out, ref, Z)
+    for wpz in (2, 4):
+        nb.burn(net, *a, *tol, kernel="coop", blob_in_shared=1, warps_per_zone=wpz)
+    with pytest.raises(nb.NetburnError):       # two zones never fitted
+        nb.burn(net, *a, *tol, kernel="coop", blob_in_shared=1, threads_per_block=64)
