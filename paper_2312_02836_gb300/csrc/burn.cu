@@ -540,8 +540,9 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
     net->last_spec = spec_variant;
     return NB_OK;
   }
+  // (a blob asked for in shared memory is the lane kernel's: it has to fit)
   if (!specialize_auto_ok(net->h) && net->h.n >= 24 && o.threads_per_block <= 0 &&
-      o.blocks_per_sm <= 0 && o.ws_in_shared <= 0) {
+      o.blocks_per_sm <= 0 && o.ws_in_shared <= 0 && o.blob_in_shared <= 0) {
     int rc = NB_OK;
     if (nb::launch_lane_teams(net, P, o, st, &rc)) return rc;
   }

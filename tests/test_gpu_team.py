@@ -289,3 +289,14 @@ def test_a_blob_and_a_zone_that_just_fit_shared_memory():
         nb.burn(net, *a, *tol, kernel="coop", blob_in_shared=1, warps_per_zone=wpz)
     with pytest.raises(nb.NetburnError):       # two zones never fitted
         nb.burn(net, *a, *tol, kernel="coop", blob_in_shared=1, threads_per_block=64)
+
+
+def test_a_large_networks_blob_asked_for_in_shared_memory():
+    # 48 species fit (the lane kernel), 128 don't
+    nb, torch, net, t, tol, sm = _setup("net48", 8, 1e-7)
+    ref = nb.burn(net, *_first(t, 8), *tol)
+    _same(torch, nb.burn(net, *_first(t, 8), *tol, blob_in_shared=1), ref, 8)
+    _, _, net, t, tol, _ = _setup("net128_heat", 8, 1e-9)
+    nb.burn(net, *_first(t, 8), *tol)
+    with pytest.raises(nb.NetburnError):
+        nb.burn(net, *_first(t, 8), *tol, blob_in_shared=1)
