@@ -429,18 +429,23 @@ int nb_burn_multi(int32_t n_sets, const nb_burn_set* sets, double t_end, double 
  * it; burns then use it as options.specialize says.  It performs the
  * generic kernel's floating-point operations in the same order, so both give
  * the same bits.
- *  variant  0: chosen from the network's sizes; 1: all Newton-loop arrays of
- *           a zone in registers; 2: as 1 with the LU in the workspace;
- *           3: only x, d, f in registers.
+ *  variant  0: every form that burns take by themselves (specialize = 0),
+ *           for whatever number of zones: variant 3 and the team forms, which
+ *           give a zone 4, 8, 16 or 32 lanes and read the compiled network
+ *           with its sizes as constants; a burn builds the one it needs
+ *           otherwise.  1: all Newton-loop arrays of a zone in registers; 2:
+ *           as 1 with the LU in the workspace; 3: only x, d, f in registers.
  *  log      NULL or a host buffer of log_bytes for the compiler's log
  *           (NUL-terminated, truncated to fit).
- * Synchronous; compiling takes seconds.  NB_E_COMPILE on failure.  A kernel
+ * Synchronous; compiling takes seconds.  NB_E_COMPILE on failure (variant 0:
+ * of variant 3; a team form that cannot be built is not used).  A kernel
  * built once is kept with the network. */
 int nb_net_specialize(nb_net net, int32_t variant, char* log, int64_t log_bytes);
 /* The specialised kernel's source for a topology, without any GPU: host
  * buffer buf of cap bytes (NUL-terminated when it fits); *len = source
  * length in bytes (without the NUL).  NB_E_ARG when cap is too small (buf
- * untouched, *len set). */
+ * untouched, *len set).  variant 0: 1, 2 or 3 by the network's sizes, the one
+ * with the most in registers that fits. */
 int nb_specialize_source(const nb_topology* topo, const double* coeffs,
                          int32_t variant, char* buf, int64_t cap, int64_t* len);
 /* Generate and compile the specialised kernel for a topology without any GPU
@@ -448,6 +453,9 @@ int nb_specialize_source(const nb_topology* topo, const double* coeffs,
  * including the register and spill report of the sm_103a assembler. */
 int nb_specialize_compile(const nb_topology* topo, const double* coeffs,
                           int32_t variant, char* log, int64_t log_bytes);
+/* The same for the team form with `lanes` (4, 8, 16 or 32) lanes per zone. */
+int nb_specialize_team_compile(const nb_topology* topo, const double* coeffs,
+                               int32_t lanes, char* log, int64_t log_bytes);
 /* The FP64 exp the rate evaluation uses (Tang's table-driven method, see
  * the kernels' expf64.cuh), and optionally the CUDA library exp, on a device
  * array x [n]: y_tang [n] (and y_lib [n] unless NULL).  A diagnostic for

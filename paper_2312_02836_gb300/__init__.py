@@ -79,13 +79,17 @@ def specialized_source(spec, variant: int = 0) -> str:
     return buf.value.decode()
 
 
-def specialize_compile(spec, variant: int = 0) -> str:
-    """Compile the specialised kernel for sm_103a without a GPU; returns the
-    compiler log (registers, spills).  Raises NetburnError on failure."""
+def specialize_compile(spec, variant: int = 0, *, lanes: int = 0) -> str:
+    """Compile the specialised kernel (lanes 4, 8, 16 or 32: its team form with
+    that many lanes per zone) for sm_103a without a GPU; returns the compiler
+    log (registers, spills).  Raises NetburnError on failure."""
     lib = _abi.load()
     arrays, topo, coef = _topology(spec)
     log = C.create_string_buffer(1 << 16)
-    rc = lib.nb_specialize_compile(C.byref(topo), coef, int(variant), log, len(log))
+    if lanes:
+        rc = lib.nb_specialize_team_compile(C.byref(topo), coef, int(lanes), log, len(log))
+    else:
+        rc = lib.nb_specialize_compile(C.byref(topo), coef, int(variant), log, len(log))
     if rc != _abi.NB_OK:
         raise NetburnError("nb_specialize_compile: " + log.value.decode(errors="replace"))
     return log.value.decode(errors="replace")
@@ -125,8 +129,8 @@ class Network:
                 if name != "reserved"}
 
     def specialize(self, variant: int = 0) -> str:
-        """Build the network-specialised kernel now (nb_net_specialize);
-        returns the compiler log."""
+        """Build the network-specialised kernel now (nb_net_specialize; variant
+        0: every form a burn takes by itself); returns the compiler log."""
         log = C.create_string_buffer(1 << 16)
         rc = _abi.load().nb_net_specialize(self.handle, int(variant), log, len(log))
         if rc != _abi.NB_OK:

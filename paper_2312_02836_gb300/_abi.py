@@ -28,7 +28,7 @@ EXPORTS = ("nb_net_load", "nb_net_free", "nb_net_get_info", "nb_default_options"
            "nb_burn_batch", "nb_burn_batch_host", "nb_tape_alloc", "nb_tape_free",
            "nb_tape_steps", "nb_tape_read", "nb_burn_adjoint", "nb_burn_adjoint_ex", "nb_burn_batch_noalloc",
            "nb_burn_multi", "nb_net_specialize", "nb_specialize_source",
-           "nb_specialize_compile",
+           "nb_specialize_compile", "nb_specialize_team_compile",
            "nb_exp_eval", "nb_zone_costs", "nb_strerror")
 
 
@@ -114,6 +114,8 @@ def load(build_if_needed: bool = True):
         lib.nb_specialize_source.restype = C.c_int
         lib.nb_specialize_compile.argtypes = [P, P, I32, P, I64]
         lib.nb_specialize_compile.restype = C.c_int
+        lib.nb_specialize_team_compile.argtypes = [P, P, I32, P, I64]
+        lib.nb_specialize_team_compile.restype = C.c_int
         lib.nb_exp_eval.argtypes = [P, P, P, I64, P]
         lib.nb_zone_costs.argtypes = [P, I64, P, P, P, D, D, D, P, P, P]
         lib.nb_zone_costs.restype = C.c_int

@@ -18,6 +18,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <thread>
 #include <vector>
 
 #include "blob.h"
@@ -265,34 +266,77 @@ int nb_net_get_info(nb_net net, nb_net_info* o) {
 // 2, 3).
 static constexpr int kBurnVariant = 3;
 
-// The specialised kernel of `variant` (an index of net->spec) for this
-// network, generated, compiled and loaded on first use.  Caller holds net->mu.
-static int spec_get(nb_net net, int variant, const void** fn) {
-  nb_net_s::Spec& sp = net->spec[variant];
+// Generate and compile form `idx` (an index of net->spec) of the specialised
+// kernel; other forms may be compiled meanwhile by other threads.
+static int spec_compile(nb_net net, int idx, std::vector<char>* cubin) noexcept {
+  try {
+    return compile_specialized(
+        idx >= nb_net_s::kSpecTeam
+            ? specialized_team_source(net->blob, 4 << (idx - nb_net_s::kSpecTeam))
+            : specialized_source(net->blob, idx),
+        cubin, &net->spec[idx].log, false);
+  } catch (...) {   // no memory for the source
+    return NB_E_COMPILE;
+  }
+}
+
+static void spec_load(nb_net net, int idx, int rc, const std::vector<char>& cubin) {
+  nb_net_s::Spec& sp = net->spec[idx];
+  if (rc == NB_OK &&
+      (cudaLibraryLoadData(&sp.lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) !=
+           cudaSuccess ||
+       cudaLibraryGetKernel(&sp.kern, sp.lib,
+                            idx >= nb_net_s::kSpecTeam ? "nb_spec_team" : "nb_spec_burn") !=
+           cudaSuccess)) {
+    cudaGetLastError();
+    if (sp.lib) cudaLibraryUnload(sp.lib);
+    sp.lib = nullptr;
+    sp.kern = nullptr;
+    sp.log += "\nloading the compiled kernel failed";
+    rc = NB_E_COMPILE;
+  }
+  sp.state = rc == NB_OK ? 1 : -1;
+}
+
+// The specialised kernel of form `idx` for this network, built on first use.
+// Caller holds net->mu.
+static int spec_get(nb_net net, int idx, const void** fn) {
+  nb_net_s::Spec& sp = net->spec[idx];
   if (sp.state == 0) {
     std::vector<char> cubin;
-    const bool team = variant >= nb_net_s::kSpecTeam;
-    const std::string src =
-        team ? specialized_team_source(net->blob, 4 << (variant - nb_net_s::kSpecTeam))
-             : specialized_source(net->blob, variant);
-    const char* name = team ? "nb_spec_team" : "nb_spec_burn";
-    int rc = compile_specialized(src, &cubin, &sp.log, false);
-    if (rc == NB_OK &&
-        (cudaLibraryLoadData(&sp.lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) !=
-             cudaSuccess ||
-         cudaLibraryGetKernel(&sp.kern, sp.lib, name) != cudaSuccess)) {
-      cudaGetLastError();
-      if (sp.lib) cudaLibraryUnload(sp.lib);
-      sp.lib = nullptr;
-      sp.kern = nullptr;
-      sp.log += "\nloading the compiled kernel failed";
-      rc = NB_E_COMPILE;
-    }
-    sp.state = rc == NB_OK ? 1 : -1;
+    const int rc = spec_compile(net, idx, &cubin);
+    spec_load(net, idx, rc, cubin);
   }
   if (sp.state != 1) return NB_E_COMPILE;
   *fn = reinterpret_cast<const void*>(sp.kern);
   return NB_OK;
+}
+
+// Build every form that burns take by themselves, for whatever number of
+// zones: one zone per lane and the teams (spec_team_lanes).  Their compilations
+// run beside one another.  Caller holds net->mu.
+static void spec_build_auto(nb_net net) {
+  constexpr int kTeams = 4;
+  const int forms[1 + kTeams] = {kBurnVariant, nb_net_s::kSpecTeam + 3, nb_net_s::kSpecTeam + 2,
+                                 nb_net_s::kSpecTeam + 1, nb_net_s::kSpecTeam};
+  const int count = 1 + kTeams - (net->h.self_heating ? 0 : 1);   // 4 lanes: self-heating only
+  std::vector<char> cubin[1 + kTeams];
+  int rc[1 + kTeams];
+  std::thread th[1 + kTeams];
+  for (int i = count - 1; i >= 0; --i) {
+    if (net->spec[forms[i]].state != 0) continue;
+    auto job = [&, i] { rc[i] = spec_compile(net, forms[i], &cubin[i]); };
+    try {
+      if (i > 0) th[i] = std::thread(job);
+      else job();
+    } catch (...) {   // no thread to be had
+      job();
+    }
+  }
+  for (int i = 0; i < count; ++i) {
+    if (th[i].joinable()) th[i].join();
+    if (net->spec[forms[i]].state == 0) spec_load(net, forms[i], rc[i], cubin[i]);
+  }
 }
 
 static void copy_log(const std::string& s, char* log, int64_t cap) {
@@ -306,6 +350,7 @@ extern "C" int nb_net_specialize(nb_net net, int32_t variant, char* log, int64_t
   if (!net || variant < 0 || variant > 3) return NB_E_ARG;
   std::lock_guard<std::mutex> lk(net->mu);
   const int v = variant > 0 ? variant : kBurnVariant;
+  if (variant == 0) spec_build_auto(net);
   const void* fn = nullptr;
   const int rc = spec_get(net, v, &fn);
   copy_log(net->spec[v].log, log, log_bytes);
@@ -342,6 +387,19 @@ extern "C" int nb_specialize_compile(const nb_topology* T, const double* coeffs,
   std::string lg;
   std::vector<char> cubin;
   rc = compile_specialized(specialized_source(blob, variant), &cubin, &lg, true);
+  copy_log(lg, log, log_bytes);
+  return rc;
+}
+
+extern "C" int nb_specialize_team_compile(const nb_topology* T, const double* coeffs,
+                                          int32_t lanes, char* log, int64_t log_bytes) {
+  if (lanes != 4 && lanes != 8 && lanes != 16 && lanes != 32) return NB_E_ARG;
+  std::vector<uint8_t> blob;
+  int rc = host_blob(T, coeffs, &blob);
+  if (rc) return rc;
+  std::string lg;
+  std::vector<char> cubin;
+  rc = compile_specialized(specialized_team_source(blob, lanes), &cubin, &lg, true);
   copy_log(lg, log, log_bytes);
   return rc;
 }

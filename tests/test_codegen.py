@@ -136,3 +136,48 @@ def test_tables_in_the_source():
     n = C.c_int64()
     assert _abi.load().nb_specialize_source(C.byref(topo), coef, 0, None, 0,
                                             C.byref(n)) == -1
+
+
+def _random_network(N, mix, heat):
+    # a random network of the sizes between the alpha chain and 48 species
+    from gen import workloads as wl
+    seed = 7
+    while True:
+        rng = np.random.Generator(np.random.PCG64(seed))
+        reac, prod = wl._random_topology(rng, N, mix)
+        if wl._connected(N, reac, prod):
+            break
+        seed += 1
+    R = reac.shape[0]
+    coeffs = wl._draw_coeffs(rng, R)
+    Q = rng.uniform(1.0, 10.0, R) if heat else None
+    return wl.NetworkSpec(name="random%d" % N, N=N, R=R, reactants=reac, products=prod,
+                          A=np.arange(1, N + 1, dtype=np.float64), coeffs=coeffs, Q=Q,
+                          self_heating=heat)
+
+
+@pytest.mark.parametrize("name,lanes", [
+    ("chain13_heat", 4), ("chain13_heat", 8), ("chain13_heat", 16), ("chain13_heat", 32),
+    ("chain13_heat_ap", 4), ("chain13_heat_scr", 16), ("chain13_heat_tab", 8),
+    ("random22", 32), ("random28", 8)])
+def test_team_forms_compile_for_sm103a(name, lanes):
+    net = (_random_network(22, (19, 32, 6), True) if name == "random22" else
+           _random_network(28, (30, 50, 10), False) if name == "random28" else
+           gen.network(name))
+    try:
+        log = nb.specialize_compile(net, lanes=lanes)
+    except nb.NetburnError as e:
+        if "libnvrtc not found" in str(e):
+            pytest.skip("no run-time compiler in this image")
+        raise
+    assert "nb_spec_team" in log and "sm_103a" in log
+    m = re.search(r"Used (\d+) registers", log)
+    assert m and int(m.group(1)) <= 255
+
+
+def test_team_form_arguments_checked():
+    arrays, topo, coef = nb._topology(gen.network("chain13"))
+    lib = _abi.load()
+    for lanes in (0, 1, 2, 12, 64):
+        assert lib.nb_specialize_team_compile(C.byref(topo), coef, lanes, None, 0) == -1
+    assert lib.nb_specialize_team_compile(None, coef, 8, None, 0) == -1

@@ -117,3 +117,26 @@ def test_specialized_watchdog():
     torch.cuda.synchronize()
     assert torch.equal(out.Y[torch.from_numpy(done).cuda()],
                        ref.Y[torch.from_numpy(done).cuda()])
+
+
+@pytest.mark.parametrize("name", ["chain13_heat", "chain13"])
+def test_a_prepared_network_compiles_nothing_more(name):
+    # after specialize() a default burn of any number of zones runs at once:
+    # the ranges of its form are the number of zones an SM gets
+    import time
+    nb, torch, net, z, s, t = _setup(name, 20000)
+    nc = nb.Network(net)
+    nc.specialize()
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    a = lambda n: [t[k][:n].contiguous() for k in ("Y", "T9", "rho")]
+    tol = (1e-9, s["rtol"], s["atol"])
+    nb.zone_costs(nc, *a(20000), *tol)
+    nb.burn(nc, *a(20000), *tol, specialize="generic")     # the device is warm
+    torch.cuda.synchronize()
+    for Z in (1, 12 * sm, 35 * sm, 58 * sm, 20000):
+        start = time.perf_counter()
+        nb.burn(nc, *a(Z), *tol)
+        torch.cuda.synchronize()
+        # a compilation takes seconds, these burns about a millisecond
+        assert time.perf_counter() - start < 0.5
+        assert nc.info()["last_specialized"] > 0
