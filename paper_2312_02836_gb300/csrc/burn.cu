@@ -460,11 +460,30 @@ static int spec_team_lanes(nb_net net, const BurnParams& P, const nb_options& o)
                                       : 0;
 }
 
+static int spec_form(int lanes) {
+  return lanes == 0 ? kBurnVariant
+                    : nb_net_s::kSpecTeam + (lanes == 4 ? 0 : lanes == 8 ? 1 : lanes == 16 ? 2 : 3);
+}
+
+// The lanes per zone of a burn under stream capture, which is no place to
+// compile and load a kernel: when the form of `lanes` has not been built, the
+// built one next to it (they give the same bits).  With none built, as outside.
+static int spec_lanes_in_capture(nb_net net, int lanes) {
+  static constexpr int kLanes[] = {0, 4, 8, 16, 32};
+  if (net->spec[spec_form(lanes)].state != 0) return lanes;
+  int want = 0, best = -1;
+  while (kLanes[want] != lanes) ++want;
+  for (int i = 0; i < 5; ++i)
+    if (net->spec[spec_form(kLanes[i])].state == 1 &&
+        (best < 0 || std::abs(i - want) < std::abs(best - want)))
+      best = i;
+  return best < 0 ? lanes : kLanes[best];
+}
+
 // Burn few zones of a network with a generated kernel on its team form (4, 8,
 // 16 or 32 lanes a zone); false when it can't be built or doesn't fit.
 static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int lanes,
                              cudaStream_t st, int* rc) {
-  const int idx = nb_net_s::kSpecTeam + (lanes == 4 ? 0 : lanes == 8 ? 1 : lanes == 16 ? 2 : 3);
   // doubles between teams: 8 mod 16, so that two teams' like accesses fall in
   // different halves of the shared-memory banks
   const int stride = (net->h.thot + net->h.tcold + 7) / 16 * 16 + 8;
@@ -474,7 +493,7 @@ static bool launch_spec_team(nb_net net, BurnParams& P, const nb_options& o, int
   while (threads > 32 && blob_b + threads / lanes * team_b > net->smem_optin) threads -= 32;
   const size_t dyn = blob_b + threads / lanes * team_b;
   const void* fn = nullptr;
-  if (dyn > net->smem_optin || spec_get(net, idx, &fn) != NB_OK) return false;
+  if (dyn > net->smem_optin || spec_get(net, spec_form(lanes), &fn) != NB_OK) return false;
   int occ = 0;
   if (nb::allow_shared(fn, net->smem_optin) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, dyn) != cudaSuccess || occ < 1) {
@@ -542,8 +561,9 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
       spec_variant = o.specialize;
     } else if (specialize_auto_ok(net->h)) {
       int rc = NB_OK;
-      if (const int lanes = spec_team_lanes(net, P, o); lanes > 0 &&
-          launch_spec_team(net, P, o, lanes, st, &rc)) {
+      int lanes = spec_team_lanes(net, P, o);
+      if (nb::capturing(st)) lanes = spec_lanes_in_capture(net, lanes);
+      if (lanes > 0 && launch_spec_team(net, P, o, lanes, st, &rc)) {
         net->last_spec = kBurnVariant;
         return rc;
       }

@@ -16,6 +16,16 @@ struct DevBuf {
   bool in_graph = false;   // a captured launch holds its address
 };
 
+// whether work on stream st is being captured into a graph
+inline bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s != cudaStreamCaptureStatusNone;
+}
+
 // Make buffer b at least `need` bytes for work on stream st.  A graph keeps
 // the addresses of its capture and may be replayed after any later call, so a
 // buffer that a capture has used is not freed when it has to grow: it goes to
@@ -23,11 +33,6 @@ struct DevBuf {
 // capture).
 template <class T>
 inline int ensure(DevBuf<T>& b, std::vector<void*>& kept, size_t need, cudaStream_t st) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    cap = cudaStreamCaptureStatusNone;
-  }
   if (!b.p || b.bytes < need) {
     if (b.p && b.in_graph) kept.push_back(b.p);
     else if (b.p) cudaFree(b.p);
@@ -37,7 +42,7 @@ inline int ensure(DevBuf<T>& b, std::vector<void*>& kept, size_t need, cudaStrea
     b.p = static_cast<T*>(p);
     b.bytes = need;
   }
-  if (cap != cudaStreamCaptureStatusNone) b.in_graph = true;
+  if (capturing(st)) b.in_graph = true;
   return NB_OK;
 }
 

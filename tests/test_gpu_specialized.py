@@ -140,3 +140,30 @@ def test_a_prepared_network_compiles_nothing_more(name):
         # a compilation takes seconds, these burns about a millisecond
         assert time.perf_counter() - start < 0.5
         assert nc.info()["last_specialized"] > 0
+
+
+@pytest.mark.parametrize("name,warm", [("chain13_heat", 3000), ("chain13_heat", 20000),
+                                       ("chain13", 1000)])
+def test_a_captured_burn_takes_a_form_that_is_built(name, warm):
+    # a burn of many zones, then the capture of one of few on the same
+    # network: another form's range, with nothing to compile
+    import time
+    nb, torch, net, z, s, t = _setup(name, warm)
+    nc = nb.Network(net)
+    a = lambda n: [t[k][:n].contiguous() for k in ("Y", "T9", "rho")]
+    tol = (1e-6, s["rtol"], s["atol"])
+    full = nb.burn(nc, *a(warm), *tol)
+    few = a(64)
+    out = nb.burn(nc, *few, *tol, specialize="generic")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    start = time.perf_counter()
+    with torch.cuda.graph(graph):
+        nb.burn(nc, *few, *tol, out=out)
+    assert time.perf_counter() - start < 1.0
+    for x in out:
+        x.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    for x, y in zip(out, full):
+        assert torch.equal(x, y[:64])
