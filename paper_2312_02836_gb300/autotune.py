@@ -40,6 +40,9 @@ GENERIC_CANDIDATES = (
     dict(specialize=-1, ws_in_shared=3, threads_per_block=96, blocks_per_sm=1),
     dict(specialize=-1, ws_in_shared=0, threads_per_block=64, blocks_per_sm=2),
     dict(specialize=-1, ws_in_shared=0, threads_per_block=128, blocks_per_sm=2),
+    # no launch shape: teams in the lane order for a network too large for a
+    # generated kernel
+    dict(specialize=-1),
 )
 
 SPECIALIZED_CANDIDATES = tuple(

@@ -108,3 +108,11 @@ def test_autotune_candidates_per_network():
     # a small network that has one: lane kernels only, generated ones included
     small = eligible(dict(specialize_auto=True, n_state=14))
     assert small == list(GENERIC_CANDIDATES) + list(SPECIALIZED_CANDIDATES)
+
+
+def test_autotune_times_the_default_launch_of_every_network():
+    # the burn without options: the generated kernel's choice, or the generic
+    # kernel without a launch shape where there is none
+    from paper_2312_02836_gb300.autotune import eligible
+    assert dict(specialize=0) in eligible(dict(specialize_auto=True, n_state=14))
+    assert dict(specialize=-1) in eligible(dict(specialize_auto=False, n_state=48))
