@@ -111,6 +111,20 @@ def coop_shape(launch):
                               launch.get("warps_per_zone", 0) or 0)
 
 
+def kernel_name(launch, info):
+    """The kernel a burn with these options ran (info: the network's, after
+    the burn)."""
+    shaped = any(launch.get(k, 0) > 0 for k in ("threads_per_block", "blocks_per_sm",
+                                                "ws_in_shared"))
+    if launch.get("kernel") == "coop":
+        return "k_burn_coop"
+    if info["last_specialized"]:
+        return "nb_spec_burn"
+    # without a launch shape a large network's zones go to teams
+    return "k_burn_coop" if info["n_state"] >= 24 and not (
+        shaped or info["specialize_auto"]) else "k_burn_persistent"
+
+
 def profiled_traffic(kernel, Z, shape, workload="chain13_heat"):
     """DRAM bytes per launch from the committed ncu summary of this kernel on
     this workload, or None when the kernel sources, the zone count or the
@@ -352,8 +366,7 @@ def run_native(args):
     local_ms = statistics.mean(ms)          # this rank's launch (its roofline)
     mean_ms = max_over_ranks(local_ms, dev)
     variant = netc.info()["last_specialized"]
-    kname = ("k_burn_coop" if launch.get("kernel") == "coop" else
-             "nb_spec_burn" if variant else "k_burn_persistent")
+    kname = kernel_name(launch, netc.info())
     counters = out.counters.cpu().numpy()
     status = out.status.cpu().numpy()
     ops = metrics.burn_ops(info, counters, net_spec.self_heating)
@@ -545,9 +558,7 @@ def config_entry(nb, torch, dev, flush, metrics, name, Z=None, steps=3, warmup=1
     done = status != 6
     ops = metrics.burn_ops(info, counters[done], net.self_heating)
     achieved = ops["flops"] / (mean_ms * 1e-3) / 1e12
-    kernel = launch.get("kernel", "persistent")
-    kname = {"coop": "k_burn_coop"}.get(kernel, "nb_spec_burn" if nc.info()["last_specialized"]
-                                        else "k_burn_persistent")
+    kname = kernel_name(launch, nc.info())
     entry = {"workload": workload_desc(name, Z), "zones": Z,
              "value": int(done.sum()) / (mean_ms * 1e-3), "unit": "zone-burns/s",
              "ms_per_step": mean_ms, "steps": steps, "launch": launch,
