@@ -300,3 +300,29 @@ def test_a_large_networks_blob_asked_for_in_shared_memory():
     nb.burn(net, *_first(t, 8), *tol)
     with pytest.raises(nb.NetburnError):
         nb.burn(net, *_first(t, 8), *tol, blob_in_shared=1)
+
+
+@pytest.mark.parametrize("N,mix,heat", [(22, (19, 32, 6), True), (28, (30, 50, 10), True),
+                                        (28, (30, 50, 10), False)])
+def test_generated_teams_of_middle_networks(N, mix, heat):
+    # networks between the chain and 48 species: fewer teams fit a block, and
+    # few of them an SM
+    import paper_2312_02836_gb300 as nb
+    import torch
+    from tests.test_codegen import _random_network
+    net = nb.Network(_random_network(N, mix, heat))
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    Z = 61 * sm
+    rng = np.random.default_rng(N)
+    Y = np.zeros((Z, N))
+    Y[:, :4] = rng.dirichlet([0.3] * 4, Z) / np.arange(1, 5)
+    log_u = lambda lo, hi: np.exp(rng.uniform(np.log(lo), np.log(hi), Z))
+    t = {k: torch.from_numpy(v).cuda()
+         for k, v in (("Y", Y), ("T9", log_u(0.5, 4.0)), ("rho", log_u(1e5, 1e7)))}
+    tol = (1e-4, 1e-8, 1e-12)
+    ref = nb.burn(net, *_first(t, Z), *tol, specialize="generic", threads_per_block=64)
+    assert int((ref.status == 0).sum()) == Z
+    for n in (1, 5 * sm, 12 * sm, 35 * sm, 60 * sm, Z):
+        out = nb.burn(net, *_first(t, n), *tol)
+        assert net.info()["last_specialized"] > 0
+        _same(torch, out, ref, n)
