@@ -442,22 +442,28 @@ int nb::schedule_longest_first(nb_net net, BurnParams& P, cudaStream_t st) {
 // take 94 ms with one lane each, 47, 39, 36 ms with 8, 16, 32. A team costs
 // an SM more instructions per zone, though, so the more zones the fewer
 // lanes: 500 zones 99 / 49 / 41 / 38 ms; 1,500 (10 an SM) 100 / 50 / 44 /
-// 67; 4,096 (27) 100 / 59 / 92 / 144. With 4 lanes 4,096 zones take 70 ms,
-// 8,192 (54) 83 where 8 lanes take 110 and one 101, 12,345 (81) 136 and 102;
-// effective rates, whose attempt is more rates, which spread: 10,007 (66) 146
-// and 158, 14,000 (92) 178 and 159. At fixed temperature an attempt is mostly
-// what doesn't spread, and 4 lanes never win (8,192 zones 54, 68, 53 ms with
-// 4, 8 and one). A launch shape asked for is a lane kernel's.
+// 67; 4,096 (27) 100 / 59 / 92 / 144. Four lanes and one (zones an SM, ms):
+// 60: 89 and 101; tabulated rates 125 and 130; effective rates, whose attempt
+// is more rates, which spread: 66: 139 and 157, 70: 155 and 157, 72: 163 and
+// 157. At fixed temperature an attempt is mostly what doesn't spread. There 8
+// lanes win while the teams of one block hold an SM's zones, 32, and no
+// longer (32: 41 ms, 33: 67; one lane 52), except in a network with more to
+// spread than the chain's 206 statements (698, of 14 species and 26 rates: 40
+// zones 57 and 95 ms; 2,051 statements 59 and 121). The lines hold from the
+// chain up to 28 species and 90 rates: at 60 zones an SM 22 self-heating
+// species take 217 ms with 4 lanes and 252 with one, 28 species 523 and 604.
+// A launch shape asked for is a lane kernel's.
 static int spec_team_lanes(nb_net net, const BurnParams& P, const nb_options& o) {
   if (o.threads_per_block > 0 || o.blocks_per_sm > 0) return 0;
   const long long sm = net->sm_count;
   const bool sh = net->h.self_heating != 0;
-  const long long four = !sh ? 0 : net->h.n_ap > 0 ? 72 : 60;
-  return P.Z <= 5 * sm                ? 32
-         : P.Z <= 12 * sm             ? 16
-         : P.Z <= (sh ? 35 : 40) * sm ? 8
-         : P.Z <= four * sm           ? 4
-                                      : 0;
+  const long long eight = sh ? 35 : straight_line_size(net->h) < 400 ? 32 : 40;
+  const long long four = !sh ? 0 : net->h.n_ap > 0 ? 68 : 60;
+  return P.Z <= 5 * sm       ? 32
+         : P.Z <= 12 * sm    ? 16
+         : P.Z <= eight * sm ? 8
+         : P.Z <= four * sm  ? 4
+                             : 0;
 }
 
 static int spec_form(int lanes) {

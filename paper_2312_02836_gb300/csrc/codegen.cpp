@@ -102,12 +102,11 @@ int resolve_variant(const BlobHeader& h, int variant) {
   return 3;
 }
 
-bool specialize_auto_ok(const BlobHeader& h) {
-  // straight-line size: RHS + Jacobian gathers, LU updates, solves
-  const long long stmts = (long long)h.n_rhs + h.n_js + h.nD + h.n_fw + h.n_bw + h.nd +
-                          2LL * h.R;
-  return stmts <= 6000;
+long long straight_line_size(const BlobHeader& h) {
+  return (long long)h.n_rhs + h.n_js + h.nD + h.n_fw + h.n_bw + h.nd + 2LL * h.R;
 }
+
+bool specialize_auto_ok(const BlobHeader& h) { return straight_line_size(h) <= 6000; }
 
 std::string specialized_source(const std::vector<uint8_t>& blob, int variant) {
   const BlobHeader& h = *reinterpret_cast<const BlobHeader*>(blob.data());

@@ -11,6 +11,10 @@ namespace nb {
 // Storage variant 1..3 for `variant`, 0 = chosen from the network's sizes.
 int resolve_variant(const BlobHeader& h, int variant);
 
+// Statements of the network's straight-line code: RHS and Jacobian gathers, LU
+// updates, solves.
+long long straight_line_size(const BlobHeader& h);
+
 // Whether the automatic choice specialises this network (its straight-line
 // code stays small enough to compile in seconds).
 bool specialize_auto_ok(const BlobHeader& h);

@@ -326,3 +326,27 @@ def test_generated_teams_of_middle_networks(N, mix, heat):
         out = nb.burn(net, *_first(t, n), *tol)
         assert net.info()["last_specialized"] > 0
         _same(torch, out, ref, n)
+
+
+def _best_ms(torch, call, n=3):
+    call()
+    ms = []
+    for _ in range(n):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        ms.append(a.elapsed_time(b))
+    return min(ms)
+
+
+@pytest.mark.parametrize("name,per_sm", [("chain13", 32), ("chain13", 33), ("chain13", 40),
+                                         ("chain13_heat", 60), ("chain13_heat_ap", 68)])
+def test_teams_are_no_slower_than_the_lanes_they_replace(name, per_sm):
+    # 15 % for the noise; teams past their line were 28 % slower
+    nb, torch, net, t, tol, sm = _setup(name, per_sm * 160)
+    a = _first(t, per_sm * sm)
+    lane = _best_ms(torch, lambda: nb.burn(net, *a, *tol, specialize=3,
+                                           threads_per_block=(per_sm + 31) // 32 * 32))
+    assert _best_ms(torch, lambda: nb.burn(net, *a, *tol)) < 1.15 * lane
