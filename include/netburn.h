@@ -390,7 +390,9 @@ int nb_burn_batch_noalloc(nb_net net, int64_t Z, const double* Y0,
  * network with its own zones and arrays (as for nb_burn_batch, device
  * pointers, [Z, N] with that network's N), in one persistent launch whose
  * device queue spans all of them: a few expensive zones of a large network
- * and many cheap zones of a small one share the GPU's lanes.  Sets of larger
+ * and many cheap zones of a small one share the GPU's lanes.  (Many zones of
+ * small networks beside a large one, without a watchdog: a launch for the
+ * large and one for the small, in this order.)  Sets of larger
  * networks are claimed first, and within a set (schedule 1, the default)
  * the zones longest first by their starting step, as nb_burn_batch orders
  * them.  Every zone follows the generic kernel, bit for bit the result

@@ -151,3 +151,40 @@ def test_watchdog_of_several_networks(Z, budget):
         assert torch.equal(a.Y[ok], b.Y[ok]) and torch.equal(a.T9[ok], b.T9[ok])
         assert bool(torch.isfinite(a.Y).all())
     assert sum(int((a.status == 6).sum()) for a in cut) > 0
+
+
+@pytest.mark.parametrize("per_sm", [39, 41, 101])
+def test_a_few_zones_of_a_large_network_beside_many_of_a_small_one(per_sm):
+    # up to 40 small zones an SM in one launch of teams, beyond in two; an
+    # empty set and a second large one among them.  The chain's zones don't
+    # take much longer than without the large network's (28 %: all of them by
+    # warps took up to four times as long).
+    nb, torch = _mods()
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    chain, _, s = _set(nb, torch, "chain13_heat", per_sm * sm)
+    big = [_set(nb, torch, "net48", 16)[0], _set(nb, torch, "net48_adjoint", 5)[0]]
+    empty = _set(nb, torch, "chain13", 0)[0]
+    sets = [big[0], empty, chain, big[1]]
+    tol = (1e-3, s["rtol"], s["atol"])
+
+    def ms(call):
+        call()
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        return a.elapsed_time(b)
+
+    outs = nb.burn_multi(sets, *tol)
+    for d, out in zip(sets, outs):
+        if d["Y0"].shape[0]:
+            _equal(out, nb.burn(d["net"], d["Y0"], d["T9"], d["rho"], *tol))
+    if per_sm > 40:
+        apart = ms(lambda: nb.burn_multi([chain], *tol)) + ms(lambda: nb.burn_multi(big, *tol))
+        assert ms(lambda: nb.burn_multi(sets, *tol)) < 1.28 * apart
+    # with a watchdog the budget is the call's: one launch
+    cut = nb.burn_multi(sets, *tol, time_budget_s=5e-3)
+    for a, b in zip(cut, outs):
+        ok = a.status == 0
+        assert torch.equal(a.Y[ok], b.Y[ok]) and bool(((a.status == 6) | ok).all())
