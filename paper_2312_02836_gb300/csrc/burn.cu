@@ -586,13 +586,17 @@ static int launch_burn(nb_net net, BurnParams& P, const nb_options& o,
     // self-heating chain, 81 an SM: 64 threads 160 ms, 96 threads 108 ms).
     // Past four warps, where every warp more slows the others, up to 5 % more
     // zones than lanes are better: the last claimed are the shortest (20,000
-    // zones, 132 an SM: 128 threads 121 ms, 160 threads 140 ms).  Past 256 an
-    // SM the kernel packs its last zones
-    // (block_done), so the most lanes are the fastest: 65,536 zones take
-    // 344 ms with 128 threads, 311 ms with 256.
+    // zones, 132 an SM: 128 threads 121 ms, 160 threads 140 ms).  At fixed
+    // temperature, where zones differ more, up to 40 % more (128, 160, 192,
+    // 256 threads; the chain at 200 zones an SM 68, 66, 73, - ms, at 256 77,
+    // 82, 79, 91; 22 species at 256 148, 152, 158, 184).  Past 256 an SM the
+    // kernel packs its last zones (block_done), so the most lanes are the
+    // fastest: 65,536 zones take 344 ms with 128 threads, 311 ms with 256.
     if (o.threads_per_block <= 0) {
       const long long per_sm = (P.Z + net->sm_count - 1) / net->sm_count;
-      const long long lanes = per_sm <= 128 ? per_sm : per_sm * 20 / 21;
+      const long long lanes = per_sm <= 128              ? per_sm
+                              : net->h.self_heating != 0 ? per_sm * 20 / 21
+                                                         : std::max(128LL, per_sm * 5 / 7);
       tpb = (int)std::min(256LL, (lanes + 31) / 32 * 32);
     }
     int occ = 0;
