@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "blob.h"
+#include "codegen.h"
 #include "coop_kernel.cuh"
 #include "host.h"
 #include "../../include/netburn.h"
@@ -105,7 +106,14 @@ bool coop_shape_fits(nb_net net, const nb_options& o, int wpz, int warps) {
 //    second (16,384 zones 237 ms, two warps 560 ms), but with few zones per
 //    SM the longest zone sets the time, and two or four warps shorten it:
 //    16 zones 100, 84, 77 ms with 1, 2, 4 warps; 912 zones 100, 84, 82 ms;
-//    2,048 zones 108, 83, 83 ms; 4,096 zones 110, 167, 168 ms.
+//    2,048 zones 108, 83, 83 ms; 4,096 zones 110, 167, 168 ms;
+//  * below 2,000 statements (the chains, 16 species: 1,462) a zone has little
+//    to give a second warp, and an SM holds two teams of four warps or four
+//    of two against eight warps: always one (self-heating chain, zones an
+//    SM: 1: 45, 45, 47 ms with 1, 2, 4 warps, 6: 52, 86, 138; 16 species at
+//    6: 79, 93, 135; 22 species, 2,737 statements, at 1: 38, 35, 35).
+// threads_per_block and blocks_per_sm count a warp a zone, however many
+// threads share one here.
 int nb::launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t st) {
   const size_t blob_b = (size_t)net->h.bytes;
   const size_t hot_team = (size_t)net->h.thot * sizeof(double);
@@ -130,7 +138,8 @@ int nb::launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t
   int T = S;
   if (hot_smem) {
     if (large) T = wpz == 1 ? 128 : 256;
-    else if (wpz == 1) T = P.Z <= 6LL * net->sm_count ? 128 : P.Z <= 16LL * net->sm_count ? 64 : 32;
+    else if (wpz == 1 && straight_line_size(net->h) >= 2000)
+      T = P.Z <= 6LL * net->sm_count ? 128 : P.Z <= 16LL * net->sm_count ? 64 : 32;
   }
   int threads = T;
   if (T == 32) {
@@ -139,8 +148,9 @@ int nb::launch_coop(nb_net net, BurnParams& P, const nb_options& o, cudaStream_t
       while (warps > 1 && fixed + (size_t)warps * hot_team > net->smem_optin) --warps;
     threads = 32 * warps;
   }
-  return launch_team(net, P, o, team_kernel(T, S, hot_smem ? 1 : 0), threads, o.blocks_per_sm,
-                     in_smem, st);
+  int bps = o.blocks_per_sm;
+  if (bps > 0 && wpz == 1) bps = nb::team_blocks(bps, warps_asked, threads / T);
+  return launch_team(net, P, o, team_kernel(T, S, hot_smem ? 1 : 0), threads, bps, in_smem, st);
 }
 
 // A persistent burn of a large network without a generated kernel by teams in

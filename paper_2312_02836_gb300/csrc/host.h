@@ -82,6 +82,13 @@ inline cudaError_t allow_shared(const void* fn, size_t smem_optin) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_optin);
 }
 
+// Blocks of `teams` zones that hold the zones of `blocks` blocks of `warps`
+// (0: four) warps with a zone each, the shape an option asks for.
+inline int team_blocks(int blocks, int warps, int teams) {
+  const long long zones = (long long)blocks * (warps > 0 ? warps : 4);
+  return (int)std::min<long long>((zones + teams - 1) / teams, 64);
+}
+
 // doubles per lane of a start-up pass (k_burn_start)
 __host__ __device__ constexpr int start_doubles(int n, int R) { return 5 * n + 2 * R + 2; }
 // its lanes, one zone each at a time: what four blocks per SM hold (one block

@@ -350,3 +350,26 @@ def test_teams_are_no_slower_than_the_lanes_they_replace(name, per_sm):
     lane = _best_ms(torch, lambda: nb.burn(net, *a, *tol, specialize=3,
                                            threads_per_block=(per_sm + 31) // 32 * 32))
     assert _best_ms(torch, lambda: nb.burn(net, *a, *tol)) < 1.15 * lane
+
+
+@pytest.mark.parametrize("name,Z", [("chain13_heat", 6), ("net48", 12)])
+def test_cooperative_shapes_hold_the_zones_they_ask_for(name, Z):
+    # small networks keep a warp a zone; an explicit shape counts a warp a zone
+    # whatever the team: all zones of an SM at once take little longer than one
+    # (in turns they took three times as long)
+    nb, torch, net, t, tol, sm = _setup(name, Z * 160, 1e-4 if name == "net48" else None)
+    a = _first(t, Z * sm)
+    hard = int(nb.burn(net, *a, *tol, kernel="coop").counters[:, :3].sum(1).argmax())
+    one = [x[hard:hard + 1].contiguous() for x in a]
+    kw = dict(kernel="coop", threads_per_block=128, blocks_per_sm=3)
+    alone = _best_ms(torch, lambda: nb.burn(net, *one, *tol, **kw))
+    assert _best_ms(torch, lambda: nb.burn(net, *a, *tol, **kw)) < 2.0 * alone
+
+
+def test_cooperative_shape_of_one_block_an_sm():
+    # 128 threads, one block: four zones an SM at a time, not one team
+    nb, torch, net, t, tol, sm = _setup("net48", 4 * 160, 1e-4)
+    a = _first(t, 4 * sm)
+    shape = lambda bps: _best_ms(torch, lambda: nb.burn(
+        net, *a, *tol, kernel="coop", threads_per_block=128, blocks_per_sm=bps))
+    assert shape(1) < 1.4 * shape(3)
