@@ -29,6 +29,7 @@
 
 #include "blob.h"
 #include "adjoint.cuh"
+#include "codegen.h"
 #include "coop_adjoint.cuh"
 #include "device.cuh"
 #include "host.h"
@@ -227,9 +228,9 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
   cudaStream_t st = (cudaStream_t)stream;
   std::lock_guard<std::mutex> lk(net->mu);
   const size_t blob_b = (size_t)h.bytes;
-  int tpb, in_smem;
-  size_t dyn;
-  long long blocks;
+  int tpb = 0, in_smem = 0;
+  size_t dyn = 0;
+  long long blocks = 0;
   CoopAdj C;
   std::memset(&C, 0, sizeof(C));
   const size_t scratch = team_scratch_bytes(64);
@@ -248,6 +249,50 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     lane_team = n >= 24 ? 64 : Z <= 12 * sm ? 32 : Z <= 24 * sm ? 16 : Z <= 160 * sm ? 8 : 0;
   }
   int teams = 1;   // zones of a block of teams
+  if (lane_team) {
+    team_layout(h, K, tp->dev.stride, 0, &C.a);
+    C.stride = (h.thot + C.a.total + 7) / 16 * 16 + 8;
+    const size_t team_b = (size_t)C.stride * sizeof(double);
+    const long long per_sm = (Z + net->sm_count - 1) / net->sm_count;
+    // a team of several warps is a block of its own (its barrier and its
+    // broadcasts are the block's)
+    tpb = lane_team > 32 ? lane_team
+                         : (int)std::min<long long>(128, (per_sm * lane_team + 31) / 32 * 32);
+    in_smem = blob_b <= 32 * 1024;
+    const size_t fixed = (in_smem ? blob_b : 0) + scratch;
+    while (lane_team <= 32 && tpb > 32 && fixed + tpb / lane_team * team_b > net->smem_optin) tpb -= 32;
+    teams = tpb / lane_team;
+    C.smem = fixed + teams * team_b <= net->smem_optin;
+    dyn = fixed + (C.smem ? teams * team_b : 0);
+    team_fn = lane_team == 8    ? &k_adjoint_coop<8, 0, 128, 2>
+              : lane_team == 16 ? &k_adjoint_coop<16, 0, 128, 2>
+              : lane_team == 32 ? &k_adjoint_coop<32, 0, 128, 2>
+                                : &k_adjoint_coop<64, 0, 64, 4>;
+    CK(nb::allow_shared((const void*)team_fn, net->smem_optin));
+    int occ = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
+    // The lane kernel holds all of an SM's zones at once; teams take them by
+    // turns, and the more K and the tape's stride fill their arrays the fewer
+    // at a time.  Its time over that of one turn of the teams (self-heating
+    // chain, 120 to 160 zones an SM): K = 1, strides 16, 64, 256: 7.4 (32
+    // resident: 368 and 550 ms), 6.5 (16: 435 and 380), 5.7 (4: 1,577 and
+    // 296); K = 6: 15; K = 16: 23, 17; in global memory, where 32 are
+    // resident, 3.7 (K = 1, stride 1,400: 267 and 261 ms), 6, 10 for K = 1,
+    // 16, 64.  Networks past the chains (349 statements) more: 16 species
+    // (1,462) 20 to 26, 19 species (1,772) and up 51 and more.  A large
+    // network's lane takes 20 to 80 times its team's time.
+    const long long size = straight_line_size(h), twice = size < 1000 ? 2 : size < 1600 ? 5 : 10;
+    const long long turns = (C.smem ? 5 + K : 3 + K / 8) * twice / 2;
+    if (occ < 1 || (lane_team <= 32 && per_sm > turns * occ * teams)) {
+      lane_team = 0;
+    } else {
+      blocks = std::min((long long)occ * net->sm_count, (Z + teams - 1) / teams);
+      per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
+      int rc = nb::ensure(net->ws_adj, net->kept,
+                          std::max<size_t>((size_t)blocks * teams * per_unit, 256), st);
+      if (rc) return rc;
+    }
+  }
   if (kernel == NB_KERNEL_COOP) {
     // per team in shared memory: the forward hot arrays and the adjoint's
     const int S = 32;
@@ -291,34 +336,7 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     const size_t need = (size_t)blocks * per_unit;
     int rc = nb::ensure(net->ws_adj, net->kept, std::max<size_t>(need, 256), st);
     if (rc) return rc;
-  } else if (lane_team) {
-    team_layout(h, K, tp->dev.stride, 0, &C.a);
-    C.stride = (h.thot + C.a.total + 7) / 16 * 16 + 8;
-    const size_t team_b = (size_t)C.stride * sizeof(double);
-    const long long per_sm = (Z + net->sm_count - 1) / net->sm_count;
-    // a team of several warps is a block of its own (its barrier and its
-    // broadcasts are the block's)
-    tpb = lane_team > 32 ? lane_team
-                         : (int)std::min<long long>(128, (per_sm * lane_team + 31) / 32 * 32);
-    in_smem = blob_b <= 32 * 1024;
-    const size_t fixed = (in_smem ? blob_b : 0) + scratch;
-    while (lane_team <= 32 && tpb > 32 && fixed + tpb / lane_team * team_b > net->smem_optin) tpb -= 32;
-    teams = tpb / lane_team;
-    C.smem = fixed + teams * team_b <= net->smem_optin;
-    dyn = fixed + (C.smem ? teams * team_b : 0);
-    team_fn = lane_team == 8    ? &k_adjoint_coop<8, 0, 128, 2>
-              : lane_team == 16 ? &k_adjoint_coop<16, 0, 128, 2>
-              : lane_team == 32 ? &k_adjoint_coop<32, 0, 128, 2>
-                                : &k_adjoint_coop<64, 0, 64, 4>;
-    CK(nb::allow_shared((const void*)team_fn, net->smem_optin));
-    int occ = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
-    if (occ < 1) return NB_E_TOO_LARGE;
-    blocks = std::min((long long)occ * net->sm_count, (Z + teams - 1) / teams);
-    per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
-    int rc = nb::ensure(net->ws_adj, net->kept, std::max<size_t>((size_t)blocks * teams * per_unit, 256), st);
-    if (rc) return rc;
-  } else {
+  } else if (!lane_team) {
     // one zone per lane; smaller blocks when there are few zones per SM
     const long long per_sm = (Z + net->sm_count - 1) / net->sm_count;
     tpb = o.threads_per_block > 0 ? o.threads_per_block

@@ -373,3 +373,22 @@ def test_cooperative_shape_of_one_block_an_sm():
     shape = lambda bps: _best_ms(torch, lambda: nb.burn(
         net, *a, *tol, kernel="coop", threads_per_block=128, blocks_per_sm=bps))
     assert shape(1) < 1.4 * shape(3)
+
+
+@pytest.mark.parametrize("K,stride,per_sm", [(1, 64, 100), (1, 256, 20), (1, 256, 60),
+                                             (9, 256, 100), (1, 1000, 100), (1, 0, 150)])
+def test_lane_adjoint_by_teams_is_no_slower_whatever_the_tape(K, stride, per_sm):
+    # a longer checkpoint stride and more cotangents leave room for fewer teams
+    # (15 % for the noise; without the rule up to five times the lanes' time)
+    nb, torch, net, t, tol, sm = _setup("chain13_heat", per_sm * 160, 1e-5)
+    Z = per_sm * sm
+    tape = nb.Tape(net, Z, 1000, stride)
+    nb.burn(net, *_first(t, Z), *tol, tape=tape)
+    rng = np.random.default_rng(4)
+    gY = torch.from_numpy(rng.normal(size=(K, Z, net.N))).cuda()
+    lane = dict(kernel="persistent", threads_per_block=max(32, per_sm // 32 * 32),
+                blocks_per_sm=2)
+    for a, b in zip(nb.adjoint(net, tape, gY), nb.adjoint(net, tape, gY, **lane)):
+        assert torch.equal(a, b)
+    ref = _best_ms(torch, lambda: nb.adjoint(net, tape, gY, **lane), 2)
+    assert _best_ms(torch, lambda: nb.adjoint(net, tape, gY), 2) < 1.15 * ref
