@@ -307,34 +307,44 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
         warps * warp_b > net->smem_optin)
       return NB_E_TOO_LARGE;
     C.smem = o.ws_in_shared != 0 && team_b + scratch <= net->smem_optin;
-    // Threads of a team (a block each): four warps while the longest zone
+    // Threads of a team: a large network's four warps while the longest zone
     // sets the time (up to 8 zones an SM: 1,024 zones of the 48-species
-    // network take 226, 220, 184 ms with 1, 2, 4 warps), else two (4,096
-    // zones: 315, 243, 411 ms); where two zones' arrays don't fit an SM's
-    // shared memory, eight
-    if (C.smem && 2 * (team_b + 1024) > net->smem_optin) {
-      tpb = 256;
-      team_fn = &k_adjoint_coop<256, 32, 256, 1>;
-    } else if (C.smem && Z <= 8LL * net->sm_count) {
-      tpb = 128;
-      team_fn = &k_adjoint_coop<128, 32, 128, 2>;
-    } else {
-      tpb = 64;
-      team_fn = &k_adjoint_coop<64, 32, 64, 4>;
+    // network take 226, 220, 184 ms with 1, 2, 4 warps), else two (K = 6, 60
+    // zones an SM: 324, 297, 403 ms; K = 1: 201, 210, 361); where two zones'
+    // arrays don't fit an SM's shared memory, eight.  Networks with a
+    // generated kernel (up to 6,000 statements) past 8 zones an SM one, of
+    // which an SM holds eight: 28 species (4,784 statements), 8 zones an SM
+    // 129, 138, 129 ms, 30 zones 170, 249, 337; and below 3,000 statements
+    // always (24 species, 2,596 statements, 8 zones an SM 58, 64, 83 ms; the
+    // self-heating chain 82, 126, 221).
+    const long long size = straight_line_size(h), sm = net->sm_count;
+    const int P = C.smem && 2 * (team_b + 1024) > net->smem_optin         ? 256
+                  : size < 3000 || (specialize_auto_ok(h) && Z > 8 * sm) ? 32
+                  : C.smem && Z <= 8 * sm                                 ? 128
+                                                                          : 64;
+    tpb = P;
+    if (P == 32) {   // several teams a block
+      tpb = (int)std::min(128LL, 32 * ((Z + sm - 1) / sm));
+      while (C.smem && tpb > 32 && scratch + tpb / 32 * team_b > net->smem_optin) tpb -= 32;
     }
+    teams = tpb / P;
+    team_fn = P == 256   ? &k_adjoint_coop<256, 32, 256, 1>
+              : P == 128 ? &k_adjoint_coop<128, 32, 128, 2>
+              : P == 64  ? &k_adjoint_coop<64, 32, 64, 4>
+                         : &k_adjoint_coop<32, 32, 128, 2>;
+    const size_t arrays_b = C.smem ? teams * team_b : 0;
     in_smem = o.blob_in_shared != 0 && blob_b <= 96 * 1024 &&
-              blob_b + scratch + (C.smem ? team_b : 0) <= net->smem_optin;
-    dyn = (in_smem ? blob_b : 0) + scratch + (C.smem ? team_b : 0);
+              blob_b + scratch + arrays_b <= net->smem_optin;
+    dyn = (in_smem ? blob_b : 0) + scratch + arrays_b;
     CK(nb::allow_shared((const void*)team_fn, net->smem_optin));
     int occ = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)team_fn, tpb, dyn));
     if (occ < 1) return NB_E_TOO_LARGE;
-    const int bps = std::max(1, std::min(o.blocks_per_sm > 0 ? o.blocks_per_sm : occ, occ));
-    blocks = (long long)bps * net->sm_count;
-    if (blocks > Z) blocks = Z;
+    const int bps = o.blocks_per_sm > 0 ? nb::team_blocks(o.blocks_per_sm, warps, teams) : occ;
+    blocks = std::min(std::min(bps, occ) * sm, (Z + teams - 1) / teams);
     per_unit = (size_t)(h.tcold + (C.smem ? 0 : C.stride)) * 8;
-    const size_t need = (size_t)blocks * per_unit;
-    int rc = nb::ensure(net->ws_adj, net->kept, std::max<size_t>(need, 256), st);
+    int rc = nb::ensure(net->ws_adj, net->kept,
+                        std::max<size_t>((size_t)blocks * teams * per_unit, 256), st);
     if (rc) return rc;
   } else if (!lane_team) {
     // one zone per lane; smaller blocks when there are few zones per SM

@@ -392,3 +392,44 @@ def test_lane_adjoint_by_teams_is_no_slower_whatever_the_tape(K, stride, per_sm)
         assert torch.equal(a, b)
     ref = _best_ms(torch, lambda: nb.adjoint(net, tape, gY, **lane), 2)
     assert _best_ms(torch, lambda: nb.adjoint(net, tape, gY), 2) < 1.15 * ref
+
+
+def test_cooperative_adjoint_of_small_networks_holds_an_sms_zones():
+    # a warp a zone: eight zones an SM take little longer than one (four warps
+    # a zone, two of them at a time: three times)
+    nb, torch, net, t, tol, sm = _setup("chain13_heat", 8 * 160, 1e-4)
+
+    def ms(Z):
+        tape = nb.Tape(net, Z, 1400)
+        nb.burn(net, *_first(t, Z), *tol, kernel="coop", tape=tape)
+        gY = torch.ones((1, Z, net.N), dtype=torch.float64, device="cuda")
+        return _best_ms(torch, lambda: nb.adjoint(net, tape, gY), 2)
+
+    assert ms(8 * sm) < 2.0 * ms(sm)
+
+
+def test_cooperative_adjoint_bits_of_a_middle_network():
+    import paper_2312_02836_gb300 as nb
+    import torch
+    from tests.test_codegen import _random_network
+    net = nb.Network(_random_network(28, (30, 50, 10), True))
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    Z, K = 8 * sm + 1, 3
+    rng = np.random.default_rng(2)
+    Y = np.zeros((Z, 28))
+    Y[:, :4] = rng.dirichlet([0.3] * 4, Z) / np.arange(1, 5)
+    log_u = lambda lo, hi: np.exp(rng.uniform(np.log(lo), np.log(hi), Z))
+    t = {k: torch.from_numpy(v).cuda()
+         for k, v in (("Y", Y), ("T9", log_u(0.5, 4.0)), ("rho", log_u(1e5, 1e7)))}
+    gY = torch.from_numpy(rng.normal(size=(K, Z, 28))).cuda()
+
+    def grads(n, **kw):
+        tape = nb.Tape(net, n, 600)
+        nb.burn(net, *_first(t, n), 1e-5, 1e-8, 1e-12, kernel="coop", tape=tape)
+        return nb.adjoint(net, tape, gY[:, :n].contiguous(), kernel="coop", **kw)
+
+    full = grads(Z)
+    for n, kw in ((8 * sm, {}), (5, {}), (Z, dict(threads_per_block=128, blocks_per_sm=1)),
+                  (Z, dict(ws_in_shared=0))):
+        for a, b in zip(grads(n, **kw), full):
+            assert torch.equal(a, b[:, :n])
