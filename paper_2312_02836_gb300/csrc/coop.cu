@@ -74,18 +74,15 @@ int launch_team(nb_net net, BurnParams& P, const nb_options& o, const TeamKernel
 
 // Whether the options' shape fits: a zone's Newton-loop arrays as the lane
 // kernels lay them out, `warps` such zones a block (0: as few as one) or one
-// with the partial sums of wpz warps, and the blob where it is asked for.
-// Teams keep a little more a zone; where that alone is too much, the arrays go
-// to the workspace.
+// with the partial sums of wpz warps, and the blob when it is asked for (left
+// to the library it stays out where it doesn't fit).  Teams keep a little more
+// a zone; where that alone is too much, the arrays go to the workspace.
 bool coop_shape_fits(nb_net net, const nb_options& o, int wpz, int warps) {
-  const size_t blob_b = (size_t)net->h.bytes, optin = net->smem_optin;
   const size_t zone_b = (size_t)net->h.hot_doubles * sizeof(double);
+  const size_t blob_b = o.blob_in_shared > 0 ? (size_t)net->h.bytes : 0;
   const size_t red = wpz > 1 ? (2 * wpz + 1) * sizeof(double) : 0;
-  const bool hot = o.ws_in_shared != 0 && zone_b + red <= optin;
-  const bool blob = o.blob_in_shared >= 0
-                        ? o.blob_in_shared != 0
-                        : blob_b <= 96 * 1024 && blob_b + (hot ? zone_b : 0) + red <= optin;
-  return (blob ? blob_b : 0) + red + (hot ? std::max(warps, 1) * zone_b : 0) <= optin;
+  const bool hot = o.ws_in_shared != 0 && zone_b + red <= net->smem_optin;
+  return blob_b + red + (hot ? std::max(warps, 1) * zone_b : 0) <= net->smem_optin;
 }
 
 }  // namespace

@@ -433,3 +433,26 @@ def test_cooperative_adjoint_bits_of_a_middle_network():
                   (Z, dict(ws_in_shared=0))):
         for a, b in zip(grads(n, **kw), full):
             assert torch.equal(a, b[:, :n])
+
+
+def test_an_explicit_cooperative_block_leaves_the_blob_out():
+    # 36 species: 96,304 bytes of compiled network, which the library keeps in
+    # shared memory by itself, and eight zones of 17,392 don't fit a block
+    # together; the zones alone do
+    import paper_2312_02836_gb300 as nb
+    import torch
+    from tests.test_codegen import _random_network
+    net = nb.Network(_random_network(36, (50, 83, 16), True))
+    Z = 100
+    rng = np.random.default_rng(6)
+    Y = np.zeros((Z, 36))
+    Y[:, :4] = rng.dirichlet([0.3] * 4, Z) / np.arange(1, 5)
+    a = [torch.from_numpy(x).cuda() for x in (Y, rng.uniform(0.5, 3.0, Z),
+                                              np.exp(rng.uniform(np.log(1e5), np.log(1e7), Z)))]
+    tol = (1e-5, 1e-8, 1e-12)
+    ref = nb.burn(net, *a, *tol, kernel="coop")
+    for kw in (dict(threads_per_block=256), dict(threads_per_block=256, blocks_per_sm=1),
+               dict(threads_per_block=32, blob_in_shared=1)):
+        _same(torch, nb.burn(net, *a, *tol, kernel="coop", **kw), ref, Z)
+    with pytest.raises(nb.NetburnError):
+        nb.burn(net, *a, *tol, kernel="coop", threads_per_block=256, blob_in_shared=1)
