@@ -313,15 +313,17 @@ extern "C" int nb_burn_adjoint_ex(nb_net net, void* tape, int32_t K, const doubl
     // zones an SM: 324, 297, 403 ms; K = 1: 201, 210, 361); where two zones'
     // arrays don't fit an SM's shared memory, eight.  Networks with a
     // generated kernel (up to 6,000 statements) past 8 zones an SM one, of
-    // which an SM holds eight: 28 species (4,784 statements), 8 zones an SM
-    // 129, 138, 129 ms, 30 zones 170, 249, 337; and below 3,000 statements
-    // always (24 species, 2,596 statements, 8 zones an SM 58, 64, 83 ms; the
-    // self-heating chain 82, 126, 221).
+    // which an SM holds eight, and with one or two cotangents always: 28
+    // species (4,784 statements), K = 1 and 6, 8 zones an SM 129 and 149 ms
+    // (four warps 129 and 141; at stride 1, K = 1, 61 and 79), 30 zones 170
+    // and 193 (two 249 and 374).  Below 3,000 statements always (24 species,
+    // 2,596 statements, 8 zones an SM 58, 64, 83 ms; the self-heating chain
+    // 82, 126, 221).
     const long long size = straight_line_size(h), sm = net->sm_count;
-    const int P = C.smem && 2 * (team_b + 1024) > net->smem_optin         ? 256
-                  : size < 3000 || (specialize_auto_ok(h) && Z > 8 * sm) ? 32
-                  : C.smem && Z <= 8 * sm                                 ? 128
-                                                                          : 64;
+    const int P = C.smem && 2 * (team_b + 1024) > net->smem_optin                     ? 256
+                  : size < 3000 || (specialize_auto_ok(h) && (Z > 8 * sm || K < 3)) ? 32
+                  : C.smem && Z <= 8 * sm                                             ? 128
+                                                                                      : 64;
     tpb = P;
     if (P == 32) {   // several teams a block
       tpb = (int)std::min(128LL, 32 * ((Z + sm - 1) / sm));
