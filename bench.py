@@ -119,7 +119,9 @@ def kernel_name(launch, info):
     if launch.get("kernel") == "coop":
         return "k_burn_coop"
     if info["last_specialized"]:
-        return "nb_spec_burn"
+        # without a shape the number of zones decides between the two forms
+        return ("nb_spec_burn" if shaped or launch.get("specialize", 0) > 0
+                else "nb_spec_team or nb_spec_burn")
     # without a launch shape a large network's zones go to teams
     return "k_burn_coop" if info["n_state"] >= 24 and not (
         shaped or info["specialize_auto"]) else "k_burn_persistent"
