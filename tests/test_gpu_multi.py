@@ -169,12 +169,15 @@ def test_a_few_zones_of_a_large_network_beside_many_of_a_small_one(per_sm):
 
     def ms(call):
         call()
-        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        a.record()
-        call()
-        b.record()
-        b.synchronize()
-        return a.elapsed_time(b)
+        best = float("inf")
+        for _ in range(3):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            call()
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
 
     outs = nb.burn_multi(sets, *tol)
     for d, out in zip(sets, outs):
